@@ -33,9 +33,9 @@ namespace jxf {
 constexpr int MAXV = 7;
 constexpr int kFluxThreads = 128;
 // minimum resident blocks of the face sweep per SM (register budget), per
-// storage type; overridable at build time for tuning sweeps
+// storage type (double: see the split weights below); overridable at build time for tuning sweeps
 #ifndef JXF_FLUX_MINB64
-#define JXF_FLUX_MINB64 1
+#define JXF_FLUX_MINB64 3
 #endif
 #ifndef JXF_FLUX_MINB32
 #define JXF_FLUX_MINB32 8
@@ -108,6 +108,8 @@ template <typename T> struct Cst {
     T B1h, B1l, B2h, B2l, dBh, dBl;
     // A = 1/(gamma-1) the same way: A1, A2 and dA = A1 - A2
     T A1h, A1l, A2h, A2l, dAh, dAl;
+    T g0l, pi0l;  // low parts of gamma0 and pinf0
+    T weno_eps4l;  // and of weno_eps4
     T mu, lam_heat, R, inv_R;
     T eps_rho, eps_rhoc2, eps_alpha, one_m_eps_alpha, weno_eps, weno_eps4;
 };
@@ -200,12 +202,14 @@ inline void fill_constants(Dev &P) {
         k.A2h = T(P.A2); k.A2l = T(P.A2 - double(k.A2h));
         k.dAh = T(P.A1 - P.A2); k.dAl = T((P.A1 - P.A2) - double(k.dAh));
         k.gamma0 = T(P.gamma0); k.pinf0 = T(P.pinf0); k.gm1_0 = T(P.gm1_0); k.gpinf0 = T(P.gpinf0);
+        k.g0l = T(P.gamma0 - double(k.gamma0)); k.pi0l = T(P.pinf0 - double(k.pinf0));
         k.mu = T(P.mu); k.lam_heat = T(P.lam_heat); k.R = T(P.R);
         k.inv_R = T(P.R > 0.0 ? 1.0 / P.R : 0.0);
         k.eps_rho = T(P.eps_rho); k.eps_rhoc2 = T(P.eps_rhoc2); k.eps_alpha = T(P.eps_alpha);
         k.one_m_eps_alpha = T(1.0 - P.eps_alpha);
         k.weno_eps = T(P.weno_eps);
         k.weno_eps4 = T(4.0 * P.weno_eps);
+        k.weno_eps4l = T(4.0 * P.weno_eps - double(k.weno_eps4));
     };
     fill(P.k64);
     fill(P.k32);
@@ -839,6 +843,295 @@ __device__ __forceinline__ void recon_face(const T (&x)[6], T eps4, T &vl, T &vr
     }
 }
 
+// --------------------------------------- double WENO5 with split weights --
+// GB300's FP64 pipe does 1.7 operations a clock and SM, its FP32 pipes 125,
+// and a conversion between the two formats takes an FP64 slot: the double
+// sweeps are bound by the FP64 pipe, and two thirds of their double
+// operations were the nonlinear weights.  The candidates of the outer
+// sub-stencils differ from the middle one by multiples of the third
+// differences T_k = D_k - 2 D_{k+1} + D_{k+2} (6 (p_0 - p_1) = -2 T_0,
+// 6 (p_2 - p_1) = -T_1), so with the normalised weights w_k of each side
+//   left value  = x2 + (D1 + 2 D2 - (2 w_0 T_0 + w_2 T_1))/6,
+//   right value = x3 - (D3 + 2 D2 - (2 w_0 T_2 + w_2 T_1))/6:
+// the weights only multiply T.  Where the stencil is resolved -- |D_k| <=
+// 2^-4 and |T_k| <= 2^-7 of the variable's scale (rho, c, rho c^2, 1) -- this
+// correction is carried in pairs of floats (an unevaluated sum hi + lo; its
+// error against exact arithmetic is 2^-50 of max |T| in the mean and 2^-45 at
+// most, so below 2^-52 of the scale and typically 2^-57): it stays below the
+// rounding of the double face value, and everything that is not
+// proportional to T (differences, middle candidate, sums) stays in double.
+// Other faces (shocks, interfaces, coarse waves) take the double formula
+// above; there the correction form would lose digits next to a jump (the
+// middle candidate's share of the jump cancels).  The choice is made per face
+// from its own stencil, so it does not depend on how faces are grouped into
+// warps.  One-dimensional grids keep the double formula for every face: they
+// are latency-bound, and a warp with a shock in it would pay for both
+// (200-cell tube: 70 against 73 us a step).
+// FP64 instructions of a 3-D viscous face: 620 -> 155; 128^3 Taylor-Green
+// step 24.8 -> 8.5 ms (sweeps 2.49 -> 0.74 ms each); right-hand sides against
+// float64 references are as close as before (1.1e-14 -> 0.9e-14 on smooth
+// 3-D fields).  Three blocks of 128 an SM (168 registers) let the integer and
+// FP32 work of one warp run beside the FP64 work of the others: 8.75 ms
+// against 9.18 with two and 9.09 with four.
+//
+// Pairs of floats, two lanes: lane x carries the left value's stencil
+// (D0..D3), lane y the mirrored one (D4..D1), as in the packed float WENO5.
+// Sums and products after Knuth / Dekker with the product error from one
+// fused multiply-add; l is not renormalised where the next operation
+// tolerates a few ulps of h in it.
+struct d2 {
+    f2 h, l;
+};
+__device__ __forceinline__ d2 bcd(float h, float l) { return {bc2(h), bc2(l)}; }
+__device__ __forceinline__ f2 neg2(f2 a) { return mul2(a, bc2(-1.f)); }
+__device__ __forceinline__ void two_sum2(f2 a, f2 b, f2 &s, f2 &e) {
+    s = add2(a, b);
+    const f2 bb = sub2(s, a);
+    e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
+}
+__device__ __forceinline__ d2 renorm(d2 a) {
+    const f2 s = add2(a.h, a.l);
+    return {s, sub2(a.l, sub2(s, a.h))};
+}
+__device__ __forceinline__ d2 dadd(d2 a, d2 b) {
+    f2 s, e;
+    two_sum2(a.h, b.h, s, e);
+    return {s, add2(e, add2(a.l, b.l))};
+}
+__device__ __forceinline__ d2 dsub(d2 a, d2 b) {
+    const f2 s = sub2(a.h, b.h);
+    const f2 bb = sub2(a.h, s);                              // what of b.h went into s
+    const f2 e = sub2(sub2(a.h, add2(s, bb)), sub2(b.h, bb));
+    return {s, add2(e, sub2(a.l, b.l))};
+}
+__device__ __forceinline__ d2 dmul(d2 a, d2 b) {
+    const f2 p = mul2(a.h, b.h);
+    const f2 r = fma2(neg2(a.h), b.h, p);  // minus the product's error
+    return {p, sub2(fma2(a.h, b.l, mul2(a.l, b.h)), r)};
+}
+__device__ __forceinline__ d2 dsq(d2 a) {
+    const f2 p = mul2(a.h, a.h);
+    const f2 r = fma2(neg2(a.h), a.h, p);
+    return {p, sub2(mul2(add2(a.h, a.h), a.l), r)};
+}
+// a times the small integer (or other exact float) c
+__device__ __forceinline__ d2 dmulf(d2 a, float c) {
+    const f2 p = mul2(a.h, bc2(c));
+    const f2 r = fma2(a.h, bc2(-c), p);
+    return {p, sub2(mul2(a.l, bc2(c)), r)};
+}
+__device__ __forceinline__ d2 dscale(d2 a, f2 s) { return {mul2(a.h, s), mul2(a.l, s)}; }  // s a power of two
+__device__ __forceinline__ d2 ddiv(d2 a, d2 b) {
+    const f2 r = rcp2(b.h);
+    const f2 q = mul2(a.h, r), nq = neg2(q);
+    const f2 rem = add2(fma2(nq, b.h, a.h), fma2(nq, b.l, a.l));
+    return {q, mul2(rem, r)};
+}
+__device__ __forceinline__ f2 swap2(f2 a) { return mk2(a.v.y, a.v.x); }
+
+// The correction 2 w_0 T_0 + w_2 T_1 of both values of a face from the
+// lanes' differences D0..D3.  The Q_k are scaled by the power of two next to
+// the largest, so that their fourth powers stay normal floats (the caller
+// bounds their spread).
+__device__ __forceinline__ d2 weno5_correction_split(bool z, d2 D0, d2 D1, d2 D2, d2 D3, float eps4,
+                                                     float eps4l) {
+    const f2 two = bc2(2.f);
+    const d2 A0 = dsub(D1, D0), A1 = dsub(D2, D1), A2 = dsub(D3, D2);
+    const d2 T0 = dsub(A1, A0), T1 = dsub(A2, A1);
+    const d2 H0 = dadd(dscale(D1, two), A0), H1 = dadd(D1, D2), H2 = dsub(A2, dscale(D2, two));
+    const f2 e4 = bc2(eps4), e4l = bc2(eps4l);
+    const float k0 = (float)(13.0 / 3.0), k1 = (float)(13.0 / 3.0 - (double)k0);
+    auto q = [&](d2 H, d2 A) {
+        const d2 h = dsq(H), a = dmul(dsq(A), bcd(k0, k1));
+        f2 s, e, t, g;
+        two_sum2(h.h, a.h, s, e);
+        two_sum2(s, e4, t, g);
+        return renorm({t, add2(add2(add2(e, g), e4l), add2(h.l, a.l))});
+    };
+    d2 Q0 = q(H0, A0), Q1 = q(H1, A1), Q2 = q(H2, A2);
+    auto pow2 = [](float m) { return __uint_as_float(0x7F000000u - (__float_as_uint(m) & 0x7F800000u)); };
+    const f2 sc = mk2(pow2(fmaxf(Q0.h.v.x, fmaxf(Q1.h.v.x, Q2.h.v.x))),
+                      pow2(fmaxf(Q0.h.v.y, fmaxf(Q1.h.v.y, Q2.h.v.y))));
+    Q0 = dscale(Q0, sc), Q1 = dscale(Q1, sc), Q2 = dscale(Q2, sc);
+    d2 num, den;
+    if (z) {
+        d2 tau = renorm(dsub(Q0, Q2));
+        const f2 sg = mk2(tau.h.v.x < 0.f ? -1.f : 1.f, tau.h.v.y < 0.f ? -1.f : 1.f);
+        tau = dscale(tau, sg);
+        const d2 p0 = renorm(dmul(renorm(dadd(Q0, tau)), Q2));
+        const d2 p1 = dmul(renorm(dadd(Q1, tau)), renorm(dmul(Q0, Q2)));
+        const d2 p2 = renorm(dmulf(dmul(renorm(dadd(Q2, tau)), Q0), 3.f));
+        num = dmul(Q1, renorm(dadd(dscale(dmul(p0, T0), two), dmul(p2, T1))));
+        den = dadd(dmul(Q1, renorm(dadd(p0, p2))), dmulf(p1, 6.f));
+    } else {
+        const d2 z0 = dsq(Q0), z1 = renorm(dsq(Q1)), z2 = renorm(dsq(Q2));
+        const d2 g = renorm(dmulf(z0, 3.f));
+        num = dmul(z1, renorm(dadd(dscale(dmul(z2, T0), two), dmul(g, T1))));
+        den = dadd(dmul(z1, renorm(dadd(z2, g))), dscale(dmul(g, z2), two));
+    }
+    return ddiv(num, renorm(den));
+}
+
+// Double to a pair of floats on the integer pipe: h the value truncated to 24
+// bits, l the remaining 29 bits rounded to float (GB300 converts between
+// double and float on the FP64 pipe, at the cost of a double operation each).
+// |x| below 2^-74 gives 0; |x| must be below 2^120 (the caller checks).
+__device__ __forceinline__ void split_double(double x, float &h, float &l) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const bool small = (hi & 0x7FFFFFFFu) < 0x3B500000u;
+    // the exponent's low 8 bits rebiased by 896 = flip of their top bit
+    const unsigned b = ((__funnelshift_l(lo, hi, 3) ^ 0x40000000u) & 0x7FFFFFFFu) | (hi & 0x80000000u);
+    const float r = (float)(int)(lo & 0x1FFFFFFFu);
+    const float scale = __uint_as_float((b & 0xFF800000u) - 0x1A000000u);  // 2^(e - 52) with x's sign
+    h = small ? 0.f : __uint_as_float(b);
+    l = small ? 0.f : r * scale;
+}
+// Float to double on the integer pipe (exact; 0 and denormals give 2^-127 or
+// a little more, far below what is added to it here).
+__device__ __forceinline__ double widen(float x) {
+    const unsigned b = __float_as_uint(x);
+    return __hiloint2double((int)((((b & 0x7FFFFFFFu) >> 3) + 0x38000000u) | (b & 0x80000000u)), (int)(b << 29));
+}
+
+constexpr float kSplitD = 1.f / 16.f;   // bound of |D| over the variable's scale
+constexpr float kSplitT = 1.f / 128.f;  // bound of |T|
+
+// Face states of a double WENO5 face by the split correction; false (nothing
+// written) where the stencil is not resolved enough for it, or its scales
+// leave the range the float pairs are normal numbers in.
+template <int MODEL, int NDIM, int d>
+__device__ __forceinline__ bool reconstruct_split(const Dev &P, const double (&S)[6][MAXV], double *WL, double *WR) {
+    using V = Vars<MODEL, NDIM>;
+    constexpr int NV = V::NV, NP = V::NP, IE = V::IE, in = NP + d;
+    const bool z = P.weno_z != 0;
+    const Cst<float> &C = P.k32;
+    const bool chr = P.recon != JXF_WENO5JS_COMP;
+    float Dh[5][NV], Dl[5][NV];
+    double E[2][NV];  // D1 + 2 D2 and D3 + 2 D2
+    float dm[NV], tm[NV];
+    unsigned top = 0;  // largest exponent word of the stencil
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+        double D[5];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) top = max(top, (unsigned)__double2hiint(S[k][v]) & 0x7FFFFFFFu);
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+            D[k] = S[k + 1][v] - S[k][v];
+            split_double(D[k], Dh[k][v], Dl[k][v]);
+        }
+        E[0][v] = 2.0 * D[2] + D[1];
+        E[1][v] = 2.0 * D[2] + D[3];
+        dm[v] = fmaxf(fmaxf(fmaxf(fabsf(Dh[0][v]), fabsf(Dh[1][v])), fmaxf(fabsf(Dh[2][v]), fabsf(Dh[3][v]))),
+                      fabsf(Dh[4][v]));
+        float t = 0.f;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) t = fmaxf(t, fabsf((Dh[k][v] - Dh[k + 1][v]) + (Dh[k + 2][v] - Dh[k + 1][v])));
+        tm[v] = t;
+    }
+    // frozen state: mean of the face's two cells, S2 + D2/2, in pairs
+    float wh[NV], wl[NV];
+    float rho = 0.f;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+        if (v < NP || v == IE || v == V::IA) split_double(S[2][v], wh[v], wl[v]);
+        if (v < NP) rho += wh[v];
+    }
+    float rc2;
+    if (MODEL == JXF_SPM) rc2 = C.gamma0 * (wh[IE] + C.pinf0);
+    else {
+        const float a1 = wh[V::IA >= 0 ? V::IA : 0];
+        rc2 = wh[IE] + (wh[IE] + (C.B2h + a1 * C.dBh)) * rcp(C.A2h + a1 * C.dAh);
+    }
+    const float c = rc2 * rsq(rho * rc2);
+    bool ok = top < 0x47600000u && rho > 1.5e-5f && rho < 1e10f && rc2 > 1.5e-5f && rc2 < 1e18f && c > 1.5e-5f;
+    // 40 max|D|^2 bounds the largest Q; the smallest is at least eps4
+    const float qlim = 7e12f * C.weno_eps4;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+        const float sc = v < NP ? rho : (v == IE ? rc2 : (v == V::IA ? 1.f : c));
+        ok = ok && dm[v] <= kSplitD * sc && tm[v] <= kSplitT * sc;
+        if (!chr) ok = ok && dm[v] * dm[v] <= qlim;
+        else ok = ok && (v == IE ? 0.01f : (kSplitD * kSplitD * 4.f) * sc * sc) <= qlim;
+    }
+    if (!ok) return false;
+
+    auto pair = [&](int k, int v) {
+        return d2{mk2(Dh[k][v], Dh[4 - k][v]), mk2(Dl[k][v], Dl[4 - k][v])};
+    };
+    auto swp = [](d2 a) { return d2{swap2(a.h), swap2(a.l)}; };
+    auto put = [&](int v, d2 o) {
+        // everything next to the cell value is small: one rounding at its size
+        WL[v] = S[2][v] + (1.0 / 6.0) * ((E[0][v] - widen(o.l.v.x)) - widen(o.h.v.x));
+        WR[v] = S[3][v] - (1.0 / 6.0) * ((E[1][v] - widen(o.l.v.y)) - widen(o.h.v.y));
+    };
+    if (!chr) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            const d2 D1 = pair(1, v);
+            put(v, weno5_correction_split(z, pair(0, v), D1, pair(2, v), swp(D1), C.weno_eps4, C.weno_eps4l));
+        }
+        return true;
+    }
+    auto mean = [&](int v) {
+        return renorm(dadd(bcd(wh[v], wl[v]), dscale(bcd(Dh[2][v], Dl[2][v]), bc2(0.5f))));
+    };
+    d2 Wk[NP];
+#pragma unroll
+    for (int k = 0; k < NP; ++k) Wk[k] = mean(k);
+    const d2 rho2 = NP == 2 ? renorm(dadd(Wk[0], Wk[NP - 1])) : Wk[0];
+    const d2 p = mean(IE);
+    d2 rc;
+    if (MODEL == JXF_SPM) {
+        rc = renorm(dmul(renorm(dadd(p, bcd(C.pinf0, C.pi0l))), bcd(C.gamma0, C.g0l)));
+    } else {
+        const d2 a1 = mean(V::IA >= 0 ? V::IA : 0);
+        const d2 A = renorm(dadd(bcd(C.A2h, C.A2l), dmul(a1, bcd(C.dAh, C.dAl))));
+        const d2 B = renorm(dadd(bcd(C.B2h, C.B2l), dmul(a1, bcd(C.dBh, C.dBl))));
+        rc = renorm(dadd(p, ddiv(renorm(dadd(p, B)), A)));
+    }
+    // t = 1/(rho c): the float estimate y and one correction y (1 - x y^2)/2
+    const d2 x = renorm(dmul(rho2, rc));
+    const f2 y = bc2(rsq(x.h.v.x));
+    const d2 xy = renorm(dmul(x, {y, bc2(0.f)}));
+    const f2 res = sub2(fma2(neg2(xy.h), y, bc2(1.f)), mul2(xy.l, y));
+    const d2 t = renorm({y, mul2(mul2(y, bc2(0.5f)), res)});
+    const d2 cb = renorm(dmul(rc, t));
+    const d2 rt = renorm(dmul(rho2, t));  // 1/c
+    const d2 irc = renorm(dmul(rt, t));   // 1/(rho c^2)
+    const f2 half = bc2(0.5f);
+    const d2 hc = dscale(rt, half), hr = dscale(irc, half);
+    // differences of the acoustic amplitudes, then of the others
+    d2 qi[3], qe[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const d2 a = dmul(hc, pair(k, in)), b = dmul(hr, pair(k, IE));
+        qe[k] = renorm(dadd(b, a));
+        qi[k] = renorm(dsub(b, a));
+    }
+    const d2 ci = weno5_correction_split(z, qi[0], qi[1], qi[2], swp(qi[1]), C.weno_eps4, C.weno_eps4l);
+    const d2 ce = weno5_correction_split(z, qe[0], qe[1], qe[2], swp(qe[1]), C.weno_eps4, C.weno_eps4l);
+    const d2 sum = renorm(dadd(ci, ce));
+    put(in, dmul(cb, renorm(dsub(ce, ci))));
+    put(IE, dmul(rc, sum));
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+        if (v == in || v == IE) continue;
+        if (v < NP) {
+            const d2 ent = renorm(dmul(Wk[v < NP ? v : 0], irc));
+            d2 q[3];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) q[k] = renorm(dsub(pair(k, v), dmul(ent, pair(k, IE))));
+            const d2 cq = weno5_correction_split(z, q[0], q[1], q[2], swp(q[1]), C.weno_eps4, C.weno_eps4l);
+            put(v, dadd(cq, dmul(Wk[v < NP ? v : 0], sum)));
+        } else {
+            const d2 D1 = pair(1, v);
+            put(v, weno5_correction_split(z, pair(0, v), D1, pair(2, v), swp(D1), C.weno_eps4, C.weno_eps4l));
+        }
+    }
+    return true;
+}
+
 // ------------------------------------------------------ reconstruction ----
 // Face states of face i+1/2 from the stencil S[j] = W_{i-2+j}, j = 0..5.
 // Characteristic mode (§3.2 steps 1-4, App. C.1): frozen state = mean of
@@ -913,11 +1206,15 @@ __device__ __forceinline__ void reconstruct_w(const Dev &P, const T (&S)[6][MAXV
 // RSV: the kernel variant's scheme family -- 0: WENO5 (Jiang-Shu or Z
 // weights, chosen per face from P.weno_z), 2: TENO6-A (its own kernels, so
 // that its registers do not weigh on the WENO5 sweeps).
+// Returns true where a double face took the split correction.
 template <typename T, int MODEL, int NDIM, int d, int RSV>
-__device__ __forceinline__ void reconstruct(const Dev &P, const T (&S)[6][MAXV], T *WL, T *WR) {
+__device__ __forceinline__ bool reconstruct(const Dev &P, const T (&S)[6][MAXV], T *WL, T *WR) {
+    if constexpr (std::is_same<T, double>::value && RSV == 0 && NDIM > 1)
+        if (reconstruct_split<MODEL, NDIM, d>(P, S, WL, WR)) return true;
     if constexpr (RSV == 2) reconstruct_w<T, MODEL, NDIM, d, 2>(P, S, WL, WR);
     else if (P.weno_z) reconstruct_w<T, MODEL, NDIM, d, 1>(P, S, WL, WR);
     else reconstruct_w<T, MODEL, NDIM, d, 0>(P, S, WL, WR);
+    return false;
 }
 
 // ------------------------------------------------------------ limiters ----
@@ -1016,6 +1313,120 @@ __device__ __forceinline__ void hllc(const Dev &P, const T *WL, const T *WR, T *
     }
 }
 
+// hllc() of a double face whose two states come from the split correction
+// (so differ by a few third differences at most): the flux of the side the
+// face lies on in double, plus its dissipative part s^{-/+} (U* - U) in float
+// pairs.  That part is a multiple of the states' jump: with mK = rho_K (s_K -
+// u_K) and a = s* - u_K = (dp - m_other du)/(mL - mR),
+//   phi = (s_K - u)/(s_K - s*) - 1 = a/(s_K - s*),
+//   U* - U = phi rho_k, phi rho w, rho (phi s* + a),
+//            phi E + a ((1 + phi) rho s* + p/(s_K - s*)), phi a1,
+// so 2^-45 of it is far below the rounding of the flux.  About 40 double
+// operations in 3-D instead of 100.  Returns false at s* = 0 (both branches
+// then enter).
+__device__ __forceinline__ f2 rsq2(f2 a) { return mk2(rsq(a.v.x), rsq(a.v.y)); }
+__device__ __forceinline__ d2 drsqrt(d2 x) {  // one correction y (1 - x y^2)/2 of the float estimate
+    const f2 y = rsq2(x.h);
+    const d2 xy = renorm(dmul(x, {y, bc2(0.f)}));
+    const f2 res = sub2(fma2(neg2(xy.h), y, bc2(1.f)), mul2(xy.l, y));
+    return renorm({y, mul2(mul2(y, bc2(0.5f)), res)});
+}
+__device__ __forceinline__ d2 droot(d2 x) {
+    const f2 y = rsq2(x.h), s = mul2(x.h, y);
+    const f2 r = add2(fma2(neg2(s), s, x.h), x.l);
+    return renorm({s, mul2(mul2(r, y), bc2(0.5f))});
+}
+__device__ __forceinline__ d2 lanes(double x, double y) {
+    float xh, xl, yh, yl;
+    split_double(x, xh, xl);
+    split_double(y, yh, yl);
+    return {mk2(xh, yh), mk2(xl, yl)};
+}
+__device__ __forceinline__ d2 swapd(d2 a) { return {swap2(a.h), swap2(a.l)}; }
+__device__ __forceinline__ d2 lane_x(d2 a) { return {bc2(a.h.v.x), bc2(a.l.v.x)}; }
+__device__ __forceinline__ d2 pick(bool y, d2 a) { return y ? bcd(a.h.v.y, a.l.v.y) : bcd(a.h.v.x, a.l.v.x); }
+
+template <int MODEL, int NDIM, int d>
+__device__ __forceinline__ bool hllc_split(const Dev &P, const double *WL, const double *WR, double *F, double &uh) {
+    using V = Vars<MODEL, NDIM>;
+    constexpr int NP = V::NP, IE = V::IE, NV = V::NV, in = NP + d;
+    const Cst<float> &C = P.k32;
+    const d2 rho = lanes(density_of<double, MODEL, NDIM>(WL), density_of<double, MODEL, NDIM>(WR));
+    const d2 u = lanes(WL[in], WR[in]), p = lanes(WL[IE], WR[IE]);
+    const d2 jump = lanes(WR[in] - WL[in], WR[IE] - WL[IE]);
+    const d2 du = lane_x(jump), dp = pick(true, jump);
+    d2 rc;
+    if (MODEL == JXF_SPM) {
+        rc = renorm(dmul(renorm(dadd(p, bcd(C.pinf0, C.pi0l))), bcd(C.gamma0, C.g0l)));
+    } else {
+        constexpr int IA = V::IA >= 0 ? V::IA : 0;
+        const d2 a1 = lanes(WL[IA], WR[IA]);
+        const d2 A = renorm(dadd(bcd(C.A2h, C.A2l), dmul(a1, bcd(C.dAh, C.dAl))));
+        const d2 B = renorm(dadd(bcd(C.B2h, C.B2l), dmul(a1, bcd(C.dBh, C.dBl))));
+        rc = renorm(dadd(p, ddiv(renorm(dadd(p, B)), A)));
+    }
+    const d2 cs = renorm(dmul(rc, drsqrt(renorm(dmul(rho, rc)))));  // c of both sides
+    const d2 c2 = renorm(dmul(cs, cs));
+    const d2 sr = droot(rho);
+    const d2 w = renorm(ddiv(sr, lane_x(renorm(dadd(sr, swapd(sr))))));  // Einfeldt weights (wL, wR)
+    const d2 wL = lane_x(w), wR = pick(true, w), c2L = lane_x(c2);
+    const d2 c2b = renorm(dadd(dadd(c2L, dmul(wR, renorm(dsub(pick(true, c2), c2L)))),
+                               dscale(dmul(renorm(dmul(wL, wR)), renorm(dsq(du))), bc2(0.5f))));
+    const d2 cb = droot(c2b);
+    // s_K - u_K: lane L min(wR du - cb, -cL), lane R max(cb - wL du, cR); the
+    // left lane is carried with its sign changed, so that both are a maximum
+    const d2 e = renorm(dsub(cb, dmul({mk2(wR.h.v.x, wL.h.v.x), mk2(wR.l.v.x, wL.l.v.x)}, du)));
+    const bool bx = e.h.v.x > cs.h.v.x || (e.h.v.x == cs.h.v.x && e.l.v.x > cs.l.v.x);
+    const bool by = e.h.v.y > cs.h.v.y || (e.h.v.y == cs.h.v.y && e.l.v.y > cs.l.v.y);
+    const f2 sgn = mk2(-1.f, 1.f);
+    const d2 su = dscale({mk2(bx ? e.h.v.x : cs.h.v.x, by ? e.h.v.y : cs.h.v.y),
+                          mk2(bx ? e.l.v.x : cs.l.v.x, by ? e.l.v.y : cs.l.v.y)}, sgn);
+    const d2 m = renorm(dmul(rho, su));
+    const d2 den = lane_x(renorm(dsub(m, swapd(m))));                       // mL - mR
+    const d2 a = renorm(ddiv(renorm(dsub(dp, dmul(swapd(m), du))), den));  // s* - u_K
+    const d2 ss = renorm(dadd(u, a));
+    const float sx = ss.h.v.x;
+    if (sx == 0.f) return false;
+    const bool right = sx < 0.f;
+    // the face's side
+    double W[MAXV], U[MAXV], rc2;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) W[v] = right ? WR[v] : WL[v];
+    prim2cons<double, MODEL, NDIM>(P, W, U, rc2);
+    const double un = W[in], pr = W[IE];
+    const d2 aK = pick(right, a), suK = pick(right, su), rK = pick(right, rho), sK = pick(right, renorm(dadd(u, su)));
+    const d2 ssK = pick(right, ss);
+    const bool sub = right ? sK.h.v.x > 0.f : sK.h.v.x < 0.f;
+    const d2 sPM = sub ? sK : bcd(0.f, 0.f);
+    const d2 dd = renorm(dsub(suK, aK));  // s_K - s*
+    // lanes (phi, p/(s_K - s*))
+    const d2 pK = pick(right, p);
+    const d2 fr = renorm(ddiv({mk2(aK.h.v.x, pK.h.v.x), mk2(aK.l.v.x, pK.l.v.x)}, dd));
+    const d2 phi = lane_x(fr), pi = pick(true, fr);
+    const d2 rs = renorm(dmul(rK, ssK));
+    const d2 ga = renorm(dmul(sPM, {mk2(phi.h.v.x, aK.h.v.x), mk2(phi.l.v.x, aK.l.v.x)}));  // sPM (phi, a)
+    const d2 g = lane_x(ga), h = pick(true, ga);
+    auto add = [&](int v, double f, d2 x) { F[v] = f + (widen(x.h.v.x) + widen(x.l.v.x)); };
+#pragma unroll
+    for (int k = 0; k < NP; ++k) {
+        const d2 r = NP == 1 ? rK : lanes(U[k], U[k]);
+        add(k, U[k] * un, dmul(g, r));
+    }
+#pragma unroll
+    for (int t = 0; t < NDIM; ++t) {
+        if (t == d) add(in, U[in] * un + pr, dmul(rK, renorm(dadd(dmul(g, ssK), h))));
+        else add(NP + t, U[NP + t] * un, dmul(g, lanes(U[NP + t], U[NP + t])));
+    }
+    const d2 q = renorm(dadd(dadd(rs, dmul(phi, rs)), pi));
+    add(IE, un * (U[IE] + pr), dadd(dmul(g, lanes(U[IE], U[IE])), dmul(h, q)));
+    if (MODEL == JXF_DIM) {
+        constexpr int IA = V::IA >= 0 ? V::IA : 0;
+        add(IA, W[IA] * un, dmul(g, lanes(W[IA], W[IA])));
+    }
+    uh = un + (widen(g.h.v.x) + widen(g.l.v.x));
+    return true;
+}
+
 // Flux-limiter test (§3.3 item 2) with the test states U_i - lam F and
 // U_{i+1} + lam F (lam = 2 D dt/dx_d); the volume fraction also carries the
 // face share of a1 div(u).  Returns true if the flux must fall back to first
@@ -1081,12 +1492,12 @@ template <typename T> __device__ __forceinline__ T thinc_psi(T a1) {
 // One face side: cell volume fractions am, ac, ap along the axis, the cell's
 // |n_d| and primitive state Wc; side 0 = the cell's upper face (WL of the
 // face), side 1 = its lower face (WR).  Leaves Wf unchanged outside
-// interface cells.
+// interface cells (returns false there).
 template <typename T, int MODEL, int NDIM>
-__device__ __forceinline__ void thinc_side(T am, T ac, T ap, T nabs, int side, const T *Wc, T *Wf) {
+__device__ __forceinline__ bool thinc_side(T am, T ac, T ap, T nabs, int side, const T *Wc, T *Wf) {
     using V = Vars<MODEL, NDIM>;
-    if (!(ac >= T(1e-4) && ac <= T(1) - T(1e-4))) return;
-    if (!((ap - ac) * (ac - am) > T(0))) return;
+    if (!(ac >= T(1e-4) && ac <= T(1) - T(1e-4))) return false;
+    if (!((ap - ac) * (ac - am) > T(0))) return false;
     const bool up = ap > am;
     const T beta = nabs + T(0.01);
     const T s = up ? T(2) * ac - T(1) : T(1) - T(2) * ac;
@@ -1097,6 +1508,7 @@ __device__ __forceinline__ void thinc_side(T am, T ac, T ap, T nabs, int side, c
     Wf[0] = a * fdiv(Wc[0], ac);
     Wf[1] = (T(1) - a) * fdiv(Wc[1], T(1) - ac);
     Wf[V::IA] = a;
+    return true;
 }
 
 // |n_d| of cell i from central differences of psi (neighbours mapped through
@@ -1574,12 +1986,13 @@ __device__ __forceinline__ void flux_face_eval(const Dev &P, double dt, const in
     T Fd[MAXV];
     if constexpr (MODEL == JXF_SPM && VH > 0) viscous_flux<T, NDIM, d, VH>(P, src, S, Fd);
     T WL[MAXV], WR[MAXV];
-    reconstruct<T, MODEL, NDIM, d, RSV>(P, S, WL, WR);
+    bool split = reconstruct<T, MODEL, NDIM, d, RSV>(P, S, WL, WR);
     if constexpr (MODEL == JXF_DIM) {
         if (P.thinc) {  // cell i's upper face value, cell i+1's lower face value
             constexpr int IA = V::IA;
-            thinc_side<T, MODEL, NDIM>(S[1][IA], S[2][IA], S[3][IA], src.nd(2), 0, S[2], WL);
-            thinc_side<T, MODEL, NDIM>(S[2][IA], S[3][IA], S[4][IA], src.nd(3), 1, S[3], WR);
+            const bool l = thinc_side<T, MODEL, NDIM>(S[1][IA], S[2][IA], S[3][IA], src.nd(2), 0, S[2], WL);
+            const bool r = thinc_side<T, MODEL, NDIM>(S[2][IA], S[3][IA], S[4][IA], src.nd(3), 1, S[3], WR);
+            split = split && !l && !r;
         }
     }
     // the lowest face of a block whose lower side is shared with the block
@@ -1589,13 +2002,17 @@ __device__ __forceinline__ void flux_face_eval(const Dev &P, double dt, const in
         int k = interp_limit<T, MODEL, NDIM>(P, WL, S[2]);
         k += interp_limit<T, MODEL, NDIM>(P, WR, S[3]);
         il_hit = counted && k != 0;
+        split = split && k == 0;
         if (k == 2 && counted) atomicAdd(P.counters, 1ull);  // count the extra side
     }
     // HLLC of the reconstructed states; the flux limiter may send the loop
     // round once more with the first-order states (one HLLC copy in code)
 #pragma unroll 1
     for (int pass = 0;; ++pass) {
-        hllc<T, MODEL, NDIM, d>(P, WL, WR, F, uh);
+        bool done = false;
+        if constexpr (std::is_same<T, double>::value && RSV == 0 && NDIM > 1)
+            if (split && pass == 0) done = hllc_split<MODEL, NDIM, d>(P, WL, WR, F, uh);
+        if (!done) hllc<T, MODEL, NDIM, d>(P, WL, WR, F, uh);
         if (pass > 0 || !P.limiter) break;
         T Ui[MAXV], Uj[MAXV];
         src.ucell(2, Ui);
