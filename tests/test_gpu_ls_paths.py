@@ -1,0 +1,84 @@
+"""The short paths of the level-set kernels against their long ones: the
+reinitialisation's float screen (results must be those of evaluating every
+cell in double, bit for bit), the geometry's one-sign cells (both kinds of a
+grid's cells against the oracle), the extension of fields that are 0 away from
+the interface and its two weight paths."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import oracle as orc  # noqa: E402
+import paper_2402_05193_gb300 as jxf  # noqa: E402
+
+P, Z, S = orc.PERIODIC, orc.ZEROGRAD, orc.SYMMETRY
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    torch.cuda.set_device(0)
+
+
+def _phi(ndim, n, h, seed, amp):
+    rng = np.random.default_rng(seed)
+    ax = np.meshgrid(*[(np.arange(n[e]) + 0.5) * h for e in reversed(range(ndim))], indexing="ij")
+    r = np.sqrt(sum((a - 0.5 * a.max()) ** 2 for a in ax))
+    phi = 0.3 * min(n) * h - r
+    return phi * (1.0 + amp * np.cos(5.0 * phi / (min(n) * h) + rng.uniform(0, 6))) + \
+        amp * 0.02 * h * rng.standard_normal(phi.shape)
+
+
+@pytest.mark.parametrize("h", [1.0 / 64, 1e-5, 3e4])
+@pytest.mark.parametrize("amp", [0.0, 0.05, 0.6])
+@pytest.mark.parametrize("ndim,n,bc", [(2, [37, 29], [(S, Z), (P, P)]), (3, [21, 17, 13], [(P, P), (Z, S), (S, S)])])
+def test_reinit_screen_is_exact(ndim, n, bc, amp, h):
+    """Zeroing by the threshold commutes with the screen: R(thr) is R(0)
+    where |R(0)| > thr and 0 elsewhere, to the last bit."""
+    grid = jxf.ls_grid(ndim, n, h, bc)
+    phi = _phi(ndim, n, h, 1, amp)
+    phi.flat[5] = 0.0
+    p = torch.from_numpy(phi).cuda()
+    full, part = torch.zeros_like(p), torch.zeros_like(p)
+    jxf.jxf_ls_reinit_rhs(grid, p, p, 0.0, full)  # threshold 0: every cell in double
+    for thr in (1e-3, 5e-2, 0.5, 2.0):
+        jxf.jxf_ls_reinit_rhs(grid, p, p, thr, part)
+        want = torch.where(full.abs() > thr, full, torch.zeros_like(full))
+        assert torch.equal(part, want), thr
+    ref = orc.ls_reinit_rhs(orc.ls_config(ndim=ndim, n=n, h=h, bc=bc), phi, phi, 5e-2)
+    jxf.jxf_ls_reinit_rhs(grid, p, p, 5e-2, part)
+    assert np.abs(part.cpu().numpy() - ref).max() < 1e-12
+
+
+def test_reinit_screen_leaves_odd_values_to_double():
+    """Values the float screen cannot hold: huge, infinite and NaN cells give
+    what the double evaluation gives, their neighbours too."""
+    grid = jxf.ls_grid(2, [40, 24], 1.0 / 40, [(Z, Z)] * 2)
+    phi = _phi(2, [40, 24], 1.0 / 40, 2, 0.05)
+    phi[3, 4], phi[10, 11], phi[17, 30] = 1e300, np.inf, np.nan
+    p = torch.from_numpy(phi).cuda()
+    full, part = torch.zeros_like(p), torch.zeros_like(p)
+    jxf.jxf_ls_reinit_rhs(grid, p, p, 0.0, full)
+    jxf.jxf_ls_reinit_rhs(grid, p, p, 5e-2, part)
+    want = torch.where(full.abs() <= 5e-2, torch.zeros_like(full), full)
+    assert torch.equal(part.isnan(), want.isnan())
+    assert torch.equal(part.nan_to_num(), want.nan_to_num())
+
+
+@pytest.mark.parametrize("steps", [1, 2, 7, 20])
+def test_extension_from_a_band(steps):
+    """Fields that are 0 away from the cut cells, odd and even step counts,
+    signed zeros and a NaN normal component among the data."""
+    n, h, bc = [23, 19, 17], 1.0 / 16, [(P, P), (Z, S), (S, Z)]
+    cfg, grid = orc.ls_config(ndim=3, n=n, h=h, bc=bc), jxf.ls_grid(3, n, h, bc)
+    phi = _phi(3, n, h, 3, 0.05)
+    _, al, dg, nr = orc.ls_geometry(cfg, phi)
+    q = np.where((al > 0) & (al < 1), np.random.default_rng(4).uniform(-1, 1, (4,) + phi.shape), 0.0)
+    q[:, 0, 0, :3] = -0.0
+    ref = orc.ls_extend(cfg, phi, q, 2, steps)
+    d = [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (phi, al, dg, nr, q)]
+    scr = torch.full((4 * phi.size,), 7.0, dtype=torch.float64, device="cuda")
+    jxf.jxf_ls_extend(grid, *d, 4, 2, steps, scr)
+    assert np.abs(d[4].cpu().numpy() - ref).max() < 1e-13
