@@ -996,6 +996,43 @@ __device__ __forceinline__ double widen(float x) {
 constexpr float kSplitD = 1.f / 16.f;   // bound of |D| over the variable's scale
 constexpr float kSplitT = 1.f / 128.f;  // bound of |T|
 
+// The frozen state of a face in float pairs: mean of its two cells, S2 + D2/2
+// (wh, wl: S2; Dh, Dl: D2), with what the projection and its inverse need.
+template <int MODEL, int NDIM> struct Frozen {
+    using V = Vars<MODEL, NDIM>;
+    static constexpr int NP = V::NP, IE = V::IE, NV = V::NV;
+    d2 W[NP];                  // (partial) densities
+    d2 rc2, c, irc2, hc, hr;  // rho c^2, c, 1/(rho c^2), 1/(2 c), 1/(2 rho c^2)
+    __device__ __forceinline__ Frozen(const Cst<float> &C, const float (&wh)[NV], const float (&wl)[NV],
+                                      const float (&Dh)[NV], const float (&Dl)[NV]) {
+        const f2 half = bc2(0.5f);
+        auto mean = [&](int v) { return renorm(dadd(bcd(wh[v], wl[v]), dscale(bcd(Dh[v], Dl[v]), half))); };
+#pragma unroll
+        for (int k = 0; k < NP; ++k) W[k] = mean(k);
+        const d2 rho = NP == 2 ? renorm(dadd(W[0], W[NP - 1])) : W[0];
+        const d2 p = mean(IE);
+        if (MODEL == JXF_SPM) {
+            rc2 = renorm(dmul(renorm(dadd(p, bcd(C.pinf0, C.pi0l))), bcd(C.gamma0, C.g0l)));
+        } else {
+            const d2 a1 = mean(V::IA >= 0 ? V::IA : 0);
+            const d2 A = renorm(dadd(bcd(C.A2h, C.A2l), dmul(a1, bcd(C.dAh, C.dAl))));
+            const d2 B = renorm(dadd(bcd(C.B2h, C.B2l), dmul(a1, bcd(C.dBh, C.dBl))));
+            rc2 = renorm(dadd(p, ddiv(renorm(dadd(p, B)), A)));
+        }
+        // t = 1/(rho c): the float estimate y and one correction y (1 - x y^2)/2
+        const d2 x = renorm(dmul(rho, rc2));
+        const f2 y = bc2(rsq(x.h.v.x));
+        const d2 xy = renorm(dmul(x, {y, bc2(0.f)}));
+        const f2 res = sub2(fma2(neg2(xy.h), y, bc2(1.f)), mul2(xy.l, y));
+        const d2 t = renorm({y, mul2(mul2(y, half), res)});
+        c = renorm(dmul(rc2, t));
+        const d2 rt = renorm(dmul(rho, t));  // 1/c
+        irc2 = renorm(dmul(rt, t));
+        hc = dscale(rt, half);
+        hr = dscale(irc2, half);
+    }
+};
+
 // Face states of a double WENO5 face by the split correction; false (nothing
 // written) where the stencil is not resolved enough for it, or its scales
 // leave the range the float pairs are normal numbers in.
@@ -1073,62 +1110,183 @@ __device__ __forceinline__ bool reconstruct_split(const Dev &P, const double (&S
         }
         return true;
     }
-    auto mean = [&](int v) {
-        return renorm(dadd(bcd(wh[v], wl[v]), dscale(bcd(Dh[2][v], Dl[2][v]), bc2(0.5f))));
-    };
-    d2 Wk[NP];
-#pragma unroll
-    for (int k = 0; k < NP; ++k) Wk[k] = mean(k);
-    const d2 rho2 = NP == 2 ? renorm(dadd(Wk[0], Wk[NP - 1])) : Wk[0];
-    const d2 p = mean(IE);
-    d2 rc;
-    if (MODEL == JXF_SPM) {
-        rc = renorm(dmul(renorm(dadd(p, bcd(C.pinf0, C.pi0l))), bcd(C.gamma0, C.g0l)));
-    } else {
-        const d2 a1 = mean(V::IA >= 0 ? V::IA : 0);
-        const d2 A = renorm(dadd(bcd(C.A2h, C.A2l), dmul(a1, bcd(C.dAh, C.dAl))));
-        const d2 B = renorm(dadd(bcd(C.B2h, C.B2l), dmul(a1, bcd(C.dBh, C.dBl))));
-        rc = renorm(dadd(p, ddiv(renorm(dadd(p, B)), A)));
-    }
-    // t = 1/(rho c): the float estimate y and one correction y (1 - x y^2)/2
-    const d2 x = renorm(dmul(rho2, rc));
-    const f2 y = bc2(rsq(x.h.v.x));
-    const d2 xy = renorm(dmul(x, {y, bc2(0.f)}));
-    const f2 res = sub2(fma2(neg2(xy.h), y, bc2(1.f)), mul2(xy.l, y));
-    const d2 t = renorm({y, mul2(mul2(y, bc2(0.5f)), res)});
-    const d2 cb = renorm(dmul(rc, t));
-    const d2 rt = renorm(dmul(rho2, t));  // 1/c
-    const d2 irc = renorm(dmul(rt, t));   // 1/(rho c^2)
-    const f2 half = bc2(0.5f);
-    const d2 hc = dscale(rt, half), hr = dscale(irc, half);
+    const Frozen<MODEL, NDIM> fz(C, wh, wl, Dh[2], Dl[2]);
     // differences of the acoustic amplitudes, then of the others
     d2 qi[3], qe[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        const d2 a = dmul(hc, pair(k, in)), b = dmul(hr, pair(k, IE));
+        const d2 a = dmul(fz.hc, pair(k, in)), b = dmul(fz.hr, pair(k, IE));
         qe[k] = renorm(dadd(b, a));
         qi[k] = renorm(dsub(b, a));
     }
     const d2 ci = weno5_correction_split(z, qi[0], qi[1], qi[2], swp(qi[1]), C.weno_eps4, C.weno_eps4l);
     const d2 ce = weno5_correction_split(z, qe[0], qe[1], qe[2], swp(qe[1]), C.weno_eps4, C.weno_eps4l);
     const d2 sum = renorm(dadd(ci, ce));
-    put(in, dmul(cb, renorm(dsub(ce, ci))));
-    put(IE, dmul(rc, sum));
+    put(in, dmul(fz.c, renorm(dsub(ce, ci))));
+    put(IE, dmul(fz.rc2, sum));
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
         if (v == in || v == IE) continue;
         if (v < NP) {
-            const d2 ent = renorm(dmul(Wk[v < NP ? v : 0], irc));
+            const d2 ent = renorm(dmul(fz.W[v < NP ? v : 0], fz.irc2));
             d2 q[3];
 #pragma unroll
             for (int k = 0; k < 3; ++k) q[k] = renorm(dsub(pair(k, v), dmul(ent, pair(k, IE))));
             const d2 cq = weno5_correction_split(z, q[0], q[1], q[2], swp(q[1]), C.weno_eps4, C.weno_eps4l);
-            put(v, dadd(cq, dmul(Wk[v < NP ? v : 0], sum)));
+            put(v, dadd(cq, dmul(fz.W[v < NP ? v : 0], sum)));
         } else {
             const d2 D1 = pair(1, v);
             put(v, weno5_correction_split(z, pair(0, v), D1, pair(2, v), swp(D1), C.weno_eps4, C.weno_eps4l));
         }
     }
+    return true;
+}
+
+// ------------------------------------------- double TENO6-A, all kept ----
+// TENO6-A's selection is sharp: where all four candidates are kept, the value
+// is the linear six-cell interpolation (1, -8, 37, 37, -8, 1)/60, the same from
+// both sides and, being linear, the same in characteristic and in primitive
+// variables.  All are kept when gamma_k >= C_T sum_j gamma_j with the largest
+// cut-off, 1e-7; gamma_k = a_k^6, a_k = 1 + tau6/(beta_k + eps) >= 1, so
+// tau6 <= 9 beta_k for every k is enough (1 >= 4e-7 10^6).  That is told in
+// float from the differences D_k: the indicators are positive definite in
+// them (no difference cancels, relative error below 2e-5, of beta_6 below
+// 6e-5), and a difference too small for float leaves beta below eps, where
+// all are kept as well.  The differences of the characteristic variables can
+// cancel (no entropy or one acoustic wave only): they are projected in float
+// pairs, and where less than 2^-30 of their terms is left the face is not
+// taken.  So a face is taken here only if the double evaluation keeps
+// everything for every variable and side; its double work is then 11
+// operations per variable instead of 260, and with equal states on both sides
+// the HLLC flux is the physical flux.  All other faces are evaluated in double
+// as before.  TENO6-A with 6th-order viscous fluxes, one right-hand side: 64^3
+// periodic vortex 3.23 -> 0.64 ms, 67x58x45 between walls (half of whose faces
+// drop stencils) 2.33 -> 1.06 ms.
+//
+// Lanes as in teno6a_pair_f2 (the mirrored differences change sign, which the
+// squares do not see).  True if both sides keep all candidates for certain.
+// D0, D1, D2: the pairs (D_0, D_4), (D_1, D_3), (D_2, D_2).
+__device__ __forceinline__ bool teno6a_keeps_all(f2 D0, f2 D1, f2 D2) {
+    const f2 D3 = swap2(D1), D4 = swap2(D0);
+    const f2 k13 = bc2((float)(13.0 / 12.0)), q = bc2(0.25f);
+    auto sq2 = [&](f2 a, f2 c) { return fma2(mul2(k13, a), a, mul2(mul2(q, c), c)); };
+    const f2 b0 = sq2(sub2(D2, D1), add2(D1, D2));
+    const f2 b1 = sq2(sub2(D3, D2), fma2(bc2(-3.f), D2, D3));
+    const f2 b2 = sq2(sub2(D1, D0), fma2(bc2(3.f), D1, neg2(D0)));
+    const f2 e1 = fma2(bc2(11.f), D2, fma2(bc2(-7.f), D3, add2(D4, D4)));
+    const f2 e2 = fma2(bc2(-2.f), D2, fma2(bc2(3.f), D3, neg2(D4)));
+    const f2 e3 = fma2(bc2(-2.f), D3, add2(D2, D4));
+    const f2 b3 = fma2(mul2(bc2((float)(1.0 / 36.0)), e1), e1,
+                       fma2(mul2(k13, e2), e2, mul2(mul2(bc2((float)(781.0 / 720.0)), e3), e3)));
+    const f2 a1 = mul2(fma2(bc2(5034.f), D2, fma2(bc2(2444.f), D1, fma2(bc2(-1636.f), D3,
+                       fma2(bc2(259.f), D4, mul2(bc2(-341.f), D0))))), bc2((float)(1.0 / 5760.0)));
+    const f2 a2 = mul2(fma2(bc2(11.f), sub2(D2, D1), sub2(D0, D3)), bc2((float)(1.0 / 16.0)));
+    const f2 a3 = mul2(fma2(bc2(-54.f), D2, fma2(bc2(40.f), D3, fma2(bc2(16.f), D1,
+                       fma2(bc2(-7.f), D4, mul2(bc2(5.f), D0))))), bc2((float)(1.0 / 144.0)));
+    const f2 a4 = mul2(fma2(bc2(3.f), sub2(D1, D2), sub2(D3, D0)), bc2((float)(1.0 / 24.0)));
+    const f2 a5 = mul2(fma2(bc2(6.f), D2, fma2(bc2(-4.f), add2(D1, D3), add2(D0, D4))), bc2((float)(1.0 / 120.0)));
+    const f2 s1 = fma2(bc2(0.25f), a3, fma2(bc2(0.0625f), a5, a1));
+    const f2 s2 = fma2(bc2((float)(63.0 / 130.0)), a4, a2);
+    const f2 s3 = fma2(bc2((float)(8825.0 / 10934.0)), a5, a3);
+    const f2 b6 = fma2(s1, s1, fma2(mul2(bc2((float)(13.0 / 3.0)), s2), s2,
+                       fma2(mul2(bc2((float)(781.0 / 20.0)), s3), s3,
+                            fma2(mul2(bc2((float)(1421461.0 / 2275.0)), a4), a4,
+                                 mul2(mul2(bc2((float)(21520059541.0 / 1377684.0)), a5), a5)))));
+    const f2 bs = mul2(fma2(bc2(4.f), b1, add2(b0, b2)), bc2((float)(1.0 / 6.0)));
+    const f2 tau = abs2(sub2(b6, bs)), tol = mul2(bc2(6e-5f), add2(b6, bs));
+    const f2 hi = add2(tau, tol);
+    // 9 less the indicators' relative error
+    const float ml = 8.5f * (fminf(fminf(b0.v.x, b1.v.x), fminf(b2.v.x, b3.v.x)) + 1e-30f);
+    const float mr = 8.5f * (fminf(fminf(b0.v.y, b1.v.y), fminf(b2.v.y, b3.v.y)) + 1e-30f);
+    return hi.v.x <= ml && hi.v.y <= mr;
+}
+
+template <int MODEL, int NDIM, int d>
+__device__ __forceinline__ bool reconstruct_central(const Dev &P, const double (&S)[6][MAXV], double *WL, double *WR) {
+    using V = Vars<MODEL, NDIM>;
+    constexpr int NV = V::NV, NP = V::NP, IE = V::IE, in = NP + d;
+    const Cst<float> &C = P.k32;
+    float Dh[5][NV], Dl[5][NV];
+    double val[NV];
+    unsigned top = 0;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+        double t[5];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) top = max(top, (unsigned)__double2hiint(S[k][v]) & 0x7FFFFFFFu);
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+            t[k] = S[k + 1][v] - S[k][v];
+            split_double(t[k], Dh[k][v], Dl[k][v]);
+        }
+        // (x2 + x3)/2 plus small terms: one rounding at the value's size
+        const double s1 = t[3] - t[1], s2 = (t[4] - t[0]) + s1;
+        val[v] = S[2][v] + (0.5 * t[2] + (1.0 / 60.0) * (s2 - 8.0 * s1));
+    }
+    bool ok = top < 0x47600000u;
+    auto pair = [&](int k, int v) {
+        return d2{mk2(Dh[k][v], Dh[4 - k][v]), mk2(Dl[k][v], Dl[4 - k][v])};
+    };
+    if (P.recon == JXF_WENO5JS_COMP) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) ok = ok && teno6a_keeps_all(pair(0, v).h, pair(1, v).h, pair(2, v).h);
+    } else {
+        float wh[NV], wl[NV], rho = 0.f;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            if (v < NP || v == IE || v == V::IA) split_double(S[2][v], wh[v], wl[v]);
+            if (v < NP) rho += wh[v];
+        }
+        float rc2;
+        if (MODEL == JXF_SPM) rc2 = C.gamma0 * (wh[IE] + C.pinf0);
+        else {
+            const float a1 = wh[V::IA >= 0 ? V::IA : 0];
+            rc2 = wh[IE] + (wh[IE] + (C.B2h + a1 * C.dBh)) * rcp(C.A2h + a1 * C.dAh);
+        }
+        ok = ok && rho > 1.5e-5f && rho < 1e10f && rc2 > 1.5e-5f && rc2 < 1e18f;
+        if (!ok) return false;
+        const Frozen<MODEL, NDIM> fz(C, wh, wl, Dh[2], Dl[2]);
+        // q = x + y (the pairs): all kept, and not cancelled beyond the pairs' accuracy
+        auto keeps = [&](const d2 (&q)[3], const f2 (&size)[3]) {
+            float m = 0.f, r = 0.f;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                m = fmaxf(m, fmaxf(fabsf(q[k].h.v.x), fabsf(q[k].h.v.y)));
+                r = fmaxf(r, fmaxf(size[k].v.x, size[k].v.y));
+            }
+            return m >= 9.3e-10f * r && teno6a_keeps_all(q[0].h, q[1].h, q[2].h);
+        };
+        d2 qi[3], qe[3];
+        f2 sz[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const d2 a = dmul(fz.hc, pair(k, in)), b = dmul(fz.hr, pair(k, IE));
+            qe[k] = renorm(dadd(b, a));
+            qi[k] = renorm(dsub(b, a));
+            sz[k] = add2(abs2(a.h), abs2(b.h));
+        }
+        ok = keeps(qe, sz) && keeps(qi, sz);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            if (v == in || v == IE) continue;
+            if (v < NP) {
+                const d2 ent = renorm(dmul(fz.W[v < NP ? v : 0], fz.irc2));
+                d2 q[3];
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    const d2 b = dmul(ent, pair(k, IE)), a = pair(k, v);
+                    q[k] = renorm(dsub(a, b));
+                    sz[k] = add2(abs2(a.h), abs2(b.h));
+                }
+                ok = ok && keeps(q, sz);
+            } else {
+                ok = ok && teno6a_keeps_all(pair(0, v).h, pair(1, v).h, pair(2, v).h);
+            }
+        }
+    }
+    if (!ok) return false;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) WL[v] = WR[v] = val[v];
     return true;
 }
 
@@ -1206,15 +1364,18 @@ __device__ __forceinline__ void reconstruct_w(const Dev &P, const T (&S)[6][MAXV
 // RSV: the kernel variant's scheme family -- 0: WENO5 (Jiang-Shu or Z
 // weights, chosen per face from P.weno_z), 2: TENO6-A (its own kernels, so
 // that its registers do not weigh on the WENO5 sweeps).
-// Returns true where a double face took the split correction.
+// Returns how a double face was reconstructed.
+enum { FACE_FULL = 0, FACE_SPLIT = 1, FACE_CENTRAL = 2 };
 template <typename T, int MODEL, int NDIM, int d, int RSV>
-__device__ __forceinline__ bool reconstruct(const Dev &P, const T (&S)[6][MAXV], T *WL, T *WR) {
+__device__ __forceinline__ int reconstruct(const Dev &P, const T (&S)[6][MAXV], T *WL, T *WR) {
     if constexpr (std::is_same<T, double>::value && RSV == 0 && NDIM > 1)
-        if (reconstruct_split<MODEL, NDIM, d>(P, S, WL, WR)) return true;
+        if (reconstruct_split<MODEL, NDIM, d>(P, S, WL, WR)) return FACE_SPLIT;
+    if constexpr (std::is_same<T, double>::value && RSV == 2)
+        if (reconstruct_central<MODEL, NDIM, d>(P, S, WL, WR)) return FACE_CENTRAL;
     if constexpr (RSV == 2) reconstruct_w<T, MODEL, NDIM, d, 2>(P, S, WL, WR);
     else if (P.weno_z) reconstruct_w<T, MODEL, NDIM, d, 1>(P, S, WL, WR);
     else reconstruct_w<T, MODEL, NDIM, d, 0>(P, S, WL, WR);
-    return false;
+    return FACE_FULL;
 }
 
 // ------------------------------------------------------------ limiters ----
@@ -1345,6 +1506,24 @@ __device__ __forceinline__ d2 lanes(double x, double y) {
 __device__ __forceinline__ d2 swapd(d2 a) { return {swap2(a.h), swap2(a.l)}; }
 __device__ __forceinline__ d2 lane_x(d2 a) { return {bc2(a.h.v.x), bc2(a.l.v.x)}; }
 __device__ __forceinline__ d2 pick(bool y, d2 a) { return y ? bcd(a.h.v.y, a.l.v.y) : bcd(a.h.v.x, a.l.v.x); }
+
+// hllc() of two equal states: the physical flux (U* = U).
+template <int MODEL, int NDIM, int d>
+__device__ __forceinline__ bool hllc_equal(const Dev &P, const double *W, double *F, double &uh) {
+    using V = Vars<MODEL, NDIM>;
+    constexpr int NP = V::NP, IE = V::IE, in = NP + d;
+    double U[MAXV], rc2;
+    prim2cons<double, MODEL, NDIM>(P, W, U, rc2);
+    const double u = W[in], p = W[IE];
+#pragma unroll
+    for (int k = 0; k < NP; ++k) F[k] = U[k] * u;
+#pragma unroll
+    for (int e = 0; e < NDIM; ++e) F[NP + e] = e == d ? U[NP + e] * u + p : U[NP + e] * u;
+    F[IE] = u * (U[IE] + p);
+    if (MODEL == JXF_DIM) F[V::IA >= 0 ? V::IA : 0] = W[V::IA >= 0 ? V::IA : 0] * u;
+    uh = u;
+    return true;
+}
 
 template <int MODEL, int NDIM, int d>
 __device__ __forceinline__ bool hllc_split(const Dev &P, const double *WL, const double *WR, double *F, double &uh) {
@@ -1986,13 +2165,13 @@ __device__ __forceinline__ void flux_face_eval(const Dev &P, double dt, const in
     T Fd[MAXV];
     if constexpr (MODEL == JXF_SPM && VH > 0) viscous_flux<T, NDIM, d, VH>(P, src, S, Fd);
     T WL[MAXV], WR[MAXV];
-    bool split = reconstruct<T, MODEL, NDIM, d, RSV>(P, S, WL, WR);
+    int how = reconstruct<T, MODEL, NDIM, d, RSV>(P, S, WL, WR);
     if constexpr (MODEL == JXF_DIM) {
         if (P.thinc) {  // cell i's upper face value, cell i+1's lower face value
             constexpr int IA = V::IA;
             const bool l = thinc_side<T, MODEL, NDIM>(S[1][IA], S[2][IA], S[3][IA], src.nd(2), 0, S[2], WL);
             const bool r = thinc_side<T, MODEL, NDIM>(S[2][IA], S[3][IA], S[4][IA], src.nd(3), 1, S[3], WR);
-            split = split && !l && !r;
+            if (l || r) how = FACE_FULL;
         }
     }
     // the lowest face of a block whose lower side is shared with the block
@@ -2002,7 +2181,7 @@ __device__ __forceinline__ void flux_face_eval(const Dev &P, double dt, const in
         int k = interp_limit<T, MODEL, NDIM>(P, WL, S[2]);
         k += interp_limit<T, MODEL, NDIM>(P, WR, S[3]);
         il_hit = counted && k != 0;
-        split = split && k == 0;
+        if (k != 0) how = FACE_FULL;
         if (k == 2 && counted) atomicAdd(P.counters, 1ull);  // count the extra side
     }
     // HLLC of the reconstructed states; the flux limiter may send the loop
@@ -2011,7 +2190,9 @@ __device__ __forceinline__ void flux_face_eval(const Dev &P, double dt, const in
     for (int pass = 0;; ++pass) {
         bool done = false;
         if constexpr (std::is_same<T, double>::value && RSV == 0 && NDIM > 1)
-            if (split && pass == 0) done = hllc_split<MODEL, NDIM, d>(P, WL, WR, F, uh);
+            if (how == FACE_SPLIT && pass == 0) done = hllc_split<MODEL, NDIM, d>(P, WL, WR, F, uh);
+        if constexpr (std::is_same<T, double>::value && RSV == 2)
+            if (how == FACE_CENTRAL && pass == 0) done = hllc_equal<MODEL, NDIM, d>(P, WL, F, uh);
         if (!done) hllc<T, MODEL, NDIM, d>(P, WL, WR, F, uh);
         if (pass > 0 || !P.limiter) break;
         T Ui[MAXV], Uj[MAXV];
