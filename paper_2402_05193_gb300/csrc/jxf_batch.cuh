@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(kCellThreads, CellMinBlocks<T>::value)
 #pragma unroll
         for (int v = 0; v < NV; ++v) U[v] = T(0);
         if (threadIdx.x < tl.count)
-            update_cell<T, MODEL, NDIM>(P, cdt, tl.start + threadIdx.x, 1, U, smax, rmin, bad);
+            update_cell<T, MODEL, NDIM>(P, cdt, tl.start + threadIdx.x, 1, epi, U, smax, rmin, bad);
         if (epi) block_partials<T, NV>(P, smax, rmin, bad, U, part + (size_t)tl.slot * (3 + MAXV));
     }
 }

@@ -111,6 +111,9 @@ template <typename T> struct Cst {
     T g0l, pi0l;  // low parts of gamma0 and pinf0
     T weno_eps4l;  // and of weno_eps4
     T mu, lam_heat, R, inv_R;
+    // viscous face flux: mu and lambda times the scales of the normal derivative
+    // and of the face interpolation
+    T mu_dn[3], mu43_dn[3], lam_dn[3], mu_fv, mu23_fv;
     T eps_rho, eps_rhoc2, eps_alpha, one_m_eps_alpha, weno_eps, weno_eps4;
 };
 
@@ -204,6 +207,14 @@ inline void fill_constants(Dev &P) {
         k.gamma0 = T(P.gamma0); k.pinf0 = T(P.pinf0); k.gm1_0 = T(P.gm1_0); k.gpinf0 = T(P.gpinf0);
         k.g0l = T(P.gamma0 - double(k.gamma0)); k.pi0l = T(P.pinf0 - double(k.pinf0));
         k.mu = T(P.mu); k.lam_heat = T(P.lam_heat); k.R = T(P.R);
+        const double fv = P.visc_half == 1 ? 0.5 : (P.visc_half == 2 ? 1.0 / 16.0 : 1.0 / 256.0);
+        for (int e = 0; e < 3; ++e) {
+            k.mu_dn[e] = T(P.mu * P.vis_dn[e]);
+            k.mu43_dn[e] = T(4.0 / 3.0 * P.mu * P.vis_dn[e]);
+            k.lam_dn[e] = T(P.lam_heat * P.vis_dn[e]);
+        }
+        k.mu_fv = T(P.mu * fv);
+        k.mu23_fv = T(2.0 / 3.0 * P.mu * fv);
         k.inv_R = T(P.R > 0.0 ? 1.0 / P.R : 0.0);
         k.eps_rho = T(P.eps_rho); k.eps_rhoc2 = T(P.eps_rhoc2); k.eps_alpha = T(P.eps_alpha);
         k.one_m_eps_alpha = T(1.0 - P.eps_alpha);
@@ -403,7 +414,7 @@ __device__ __forceinline__ void prim2cons(const Dev &P, const T *W, T *U, T &rc2
 // without the float cancellation of rho e - B).
 template <typename C, typename T, int MODEL, int NDIM>
 __device__ __forceinline__ void cons2prim(const Dev &P, const T *U, T *W, C &rho_o, C &p_o,
-                                          C &rc2_o) {
+                                          C &rc2_o, C *ir_o = nullptr) {
     using V = Vars<MODEL, NDIM>;
     const C rho = (MODEL == JXF_DIM) ? C(U[0]) + C(U[1]) : C(U[0]);
     const C ir = rcp(rho);
@@ -424,6 +435,7 @@ __device__ __forceinline__ void cons2prim(const Dev &P, const T *U, T *W, C &rho
     rho_o = rho;
     p_o = p;
     rc2_o = eos.rc2_from_p(P, p);
+    if (ir_o) *ir_o = ir;
 }
 
 // ------------------------------------------------------------ WENO5 -------
@@ -857,9 +869,10 @@ __device__ __forceinline__ void recon_face(const T (&x)[6], T eps4, T &vl, T &vr
 // 2^-4 and |T_k| <= 2^-7 of the variable's scale (rho, c, rho c^2, 1) -- this
 // correction is carried in pairs of floats (an unevaluated sum hi + lo; its
 // error against exact arithmetic is 2^-50 of max |T| in the mean and 2^-45 at
-// most, so below 2^-52 of the scale and typically 2^-57): it stays below the
-// rounding of the double face value, and everything that is not
-// proportional to T (differences, middle candidate, sums) stays in double.
+// most, so below 2^-52 of the scale and typically 2^-57), and so is its sum
+// with D1 + 2 D2 (2^-50 of |D| in the mean): together below the rounding of
+// the double face value.  The differences themselves and the sum with the
+// cell value are double.
 // Other faces (shocks, interfaces, coarse waves) take the double formula
 // above; there the correction form would lose digits next to a jump (the
 // middle candidate's share of the jump cancels).  The choice is made per face
@@ -1044,21 +1057,14 @@ __device__ __forceinline__ bool reconstruct_split(const Dev &P, const double (&S
     const Cst<float> &C = P.k32;
     const bool chr = P.recon != JXF_WENO5JS_COMP;
     float Dh[5][NV], Dl[5][NV];
-    double E[2][NV];  // D1 + 2 D2 and D3 + 2 D2
     float dm[NV], tm[NV];
     unsigned top = 0;  // largest exponent word of the stencil
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-        double D[5];
 #pragma unroll
         for (int k = 0; k < 6; ++k) top = max(top, (unsigned)__double2hiint(S[k][v]) & 0x7FFFFFFFu);
 #pragma unroll
-        for (int k = 0; k < 5; ++k) {
-            D[k] = S[k + 1][v] - S[k][v];
-            split_double(D[k], Dh[k][v], Dl[k][v]);
-        }
-        E[0][v] = 2.0 * D[2] + D[1];
-        E[1][v] = 2.0 * D[2] + D[3];
+        for (int k = 0; k < 5; ++k) split_double(S[k + 1][v] - S[k][v], Dh[k][v], Dl[k][v]);
         dm[v] = fmaxf(fmaxf(fmaxf(fabsf(Dh[0][v]), fabsf(Dh[1][v])), fmaxf(fabsf(Dh[2][v]), fabsf(Dh[3][v]))),
                       fabsf(Dh[4][v]));
         float t = 0.f;
@@ -1098,9 +1104,12 @@ __device__ __forceinline__ bool reconstruct_split(const Dev &P, const double (&S
     };
     auto swp = [](d2 a) { return d2{swap2(a.h), swap2(a.l)}; };
     auto put = [&](int v, d2 o) {
-        // everything next to the cell value is small: one rounding at its size
-        WL[v] = S[2][v] + (1.0 / 6.0) * ((E[0][v] - widen(o.l.v.x)) - widen(o.h.v.x));
-        WR[v] = S[3][v] - (1.0 / 6.0) * ((E[1][v] - widen(o.l.v.y)) - widen(o.h.v.y));
+        // D1 + 2 D2 less the correction is small next to the cell value: kept
+        // in pairs until the sum with it
+        const d2 D2 = pair(2, v);
+        const d2 e = renorm(dsub(dadd(pair(1, v), dscale(D2, bc2(2.f))), o));
+        WL[v] = fma(1.0 / 6.0, widen(e.h.v.x), fma(1.0 / 6.0, widen(e.l.v.x), S[2][v]));
+        WR[v] = fma(-1.0 / 6.0, widen(e.h.v.y), fma(-1.0 / 6.0, widen(e.l.v.y), S[3][v]));
     };
     if (!chr) {
 #pragma unroll
@@ -1996,6 +2005,77 @@ __global__ void __launch_bounds__(kCellThreads, kAuxCells == 4 ? 4 : 6) k_aux_ve
 // stencil primitives (cells i-2..i+3, boundary-mapped along d, the mirrored
 // normal velocity already flipped); src gives the temperature and the
 // cell-centred derivatives of those cells.
+// The same in double, where every operation counts: normal derivatives and
+// face velocities from the differences D_k the reconstruction forms anyway,
+//   normal derivative: D2 | 26 D2 - (D1 + D3) |
+//       2134 D2 - 116 (D1 + D3) + 9 (D0 + D4)
+//   face value: m | m - s1/16 | m + (3 s2 - 25 s1)/256,  m = x2 + D2/2,
+//       s1 = D3 - D1, s2 = (D4 - D0) + s1,
+// with mu, lambda and the scales folded into constants (43 double operations
+// per 3-D face at order 4, 60 in the form below).
+template <int H> __device__ __forceinline__ double dn_diff(const double (&D)[5]) {
+    if constexpr (H == 1) return D[2];
+    else if constexpr (H == 2) return fma(26.0, D[2], -(D[1] + D[3]));
+    else return fma(2134.0, D[2], fma(-116.0, D[1] + D[3], 9.0 * (D[0] + D[4])));
+}
+template <int H> __device__ __forceinline__ double val_diff(double x2, const double (&D)[5]) {
+    const double m = fma(0.5, D[2], x2);
+    if constexpr (H == 1) return m;
+    const double s1 = D[3] - D[1];
+    if constexpr (H == 2) return fma(-1.0 / 16.0, s1, m);
+    return fma(1.0 / 256.0, fma(3.0, (D[4] - D[0]) + s1, -25.0 * s1), m);
+}
+// 2, 16 or 256 times the face value of v[0..2H-1]
+template <int H> __device__ __forceinline__ double val_raw(const double *v) {
+    if constexpr (H == 1) return v[0] + v[1];
+    else if constexpr (H == 2) return fma(9.0, v[1] + v[2], -(v[0] + v[3]));
+    else return fma(150.0, v[2] + v[3], fma(-25.0, v[1] + v[4], 3.0 * (v[0] + v[5])));
+}
+template <int NDIM, int d, int H, typename Src>
+__device__ __forceinline__ void viscous_flux_double(const Dev &P, const Src &src, const double (&S)[6][MAXV],
+                                                    double *Fd) {
+    const Cst<double> &C = P.k64;
+    constexpr int j0 = 3 - H;
+    double dn[NDIM + 1], fu[NDIM];
+#pragma unroll
+    for (int f = 0; f < NDIM; ++f) {
+        double D[5];
+#pragma unroll
+        for (int k = 0; k < 5; ++k) D[k] = S[k + 1][1 + f] - S[k][1 + f];
+        dn[f] = dn_diff<H>(D);
+        fu[f] = val_diff<H>(S[2][1 + f], D);
+    }
+    {
+        double t[6] = {0, 0, 0, 0, 0, 0}, D[5];
+#pragma unroll
+        for (int m = 0; m < 2 * H; ++m) t[j0 + m] = src.tt(j0 + m);
+#pragma unroll
+        for (int k = 0; k < 5; ++k) D[k] = t[k + 1] - t[k];
+        dn[NDIM] = dn_diff<H>(D);
+    }
+    double work = 0.0;
+    Fd[0] = 0.0;
+#pragma unroll
+    for (int k = 0; k < NDIM; ++k) {
+        double gm[2 * H], tau;
+        if (k == d) {
+            tau = C.mu43_dn[d] * dn[d];
+            if constexpr (NDIM > 1) {
+#pragma unroll
+                for (int m = 0; m < 2 * H; ++m) gm[m] = src.gdiv(j0 + m);
+                tau = fma(-C.mu23_fv, val_raw<H>(gm), tau);
+            }
+        } else {
+#pragma unroll
+            for (int m = 0; m < 2 * H; ++m) gm[m] = src.gt(k, j0 + m);
+            tau = fma(C.mu_fv, val_raw<H>(gm), C.mu_dn[d] * dn[k]);
+        }
+        Fd[1 + k] = tau;
+        work = fma(fu[k], tau, work);
+    }
+    Fd[1 + NDIM] = fma(C.lam_dn[d], dn[NDIM], work);  // - q_d = + lambda dT/dx_d
+}
+
 template <typename T, int NDIM, int d, int H, typename Src>
 __device__ __forceinline__ void viscous_flux(const Dev &P, const Src &src, const T (&S)[6][MAXV], T *Fd) {
     const Cst<T> &C = cst<T>(P);
@@ -2163,7 +2243,10 @@ __device__ __forceinline__ void flux_face_eval(const Dev &P, double dt, const in
     }
     // dissipative flux first, while the stencil's velocities are at hand
     T Fd[MAXV];
-    if constexpr (MODEL == JXF_SPM && VH > 0) viscous_flux<T, NDIM, d, VH>(P, src, S, Fd);
+    if constexpr (MODEL == JXF_SPM && VH > 0) {
+        if constexpr (std::is_same<T, double>::value) viscous_flux_double<NDIM, d, VH>(P, src, S, Fd);
+        else viscous_flux<T, NDIM, d, VH>(P, src, S, Fd);
+    }
     T WL[MAXV], WR[MAXV];
     int how = reconstruct<T, MODEL, NDIM, d, RSV>(P, S, WL, WR);
     if constexpr (MODEL == JXF_DIM) {
@@ -2437,7 +2520,7 @@ __device__ __forceinline__ void two_sum_f(float a, float b, float &s, float &e) 
 // Velocities and the sound speed are plain float.
 template <typename T, int MODEL, int NDIM>
 __device__ __forceinline__ void cons2prim_stiff_float(const Dev &P, const T *U, T *W, T &rho_o, T &p_o,
-                                                      T &rc2_o) {
+                                                      T &rc2_o, T &ir_o) {
     using V = Vars<MODEL, NDIM>;
     static_assert(sizeof(T) == 4, "float states only");
     T rh, rl = T(0);  // density as rh + rl
@@ -2497,6 +2580,7 @@ __device__ __forceinline__ void cons2prim_stiff_float(const Dev &P, const T *U, 
     rho_o = rh;
     p_o = p;
     rc2_o = p + (p + Bh) * invA;
+    ir_o = ir;
 }
 
 // Per-block partials of the cell epilogue: [smax, rmin, bad, sums...] with
@@ -2541,39 +2625,40 @@ __device__ __forceinline__ void block_partials(const Dev &P, T smax, T rmin, boo
     }
 }
 
-// Primitives (+ temperature) of one new cell state, and its CFL rate,
-// density and admissibility for the epilogue.  Float storage recovers the
+// Primitives (+ temperature) of one new cell state and, where the epilogue
+// asks for them (epi; the first two stages do not: 25 of the update's 100
+// double operations), its CFL rate, density and admissibility.  Float storage recovers the
 // stiffened-gas pressure in double (the cancellation of rho e - B); all else
 // stays in the storage type.
 template <typename T, int MODEL, int NDIM>
-__device__ __forceinline__ void finish_cell(const Dev &P, long long i, const T *U, T &s_out,
+__device__ __forceinline__ void finish_cell(const Dev &P, long long i, const T *U, int epi, T &s_out,
                                             T &rho_out, bool &bad) {
     using V = Vars<MODEL, NDIM>;
     constexpr int NV = V::NV;
-    T Wn[MAXV], rho, p, rc2;
+    T Wn[MAXV], rho, p, rc2, ir;
     if constexpr (sizeof(T) == 4) {
-        if (P.stiff) cons2prim_stiff_float<T, MODEL, NDIM>(P, U, Wn, rho, p, rc2);
-        else cons2prim<T, T, MODEL, NDIM>(P, U, Wn, rho, p, rc2);
+        if (P.stiff) cons2prim_stiff_float<T, MODEL, NDIM>(P, U, Wn, rho, p, rc2, ir);
+        else cons2prim<T, T, MODEL, NDIM>(P, U, Wn, rho, p, rc2, &ir);
     } else {
-        cons2prim<T, T, MODEL, NDIM>(P, U, Wn, rho, p, rc2);
+        cons2prim<T, T, MODEL, NDIM>(P, U, Wn, rho, p, rc2, &ir);
     }
     T *Wo = static_cast<T *>(P.Wout);
     const size_t nc = (size_t)P.vstride;
     const int ic = (int)i;  // below 2^31 (checked at creation)
 #pragma unroll
     for (int v = 0; v < NV; ++v) (Wo + v * nc)[ic] = Wn[v];
-    // one reciprocal square root t = 1/(rho c): c = rho c^2 t, 1/rho = rho c^2 t^2
-    const T t = rsq(rho * rc2);
-    const T cs = rc2 * t;
-    if (MODEL == JXF_SPM && P.viscous)
-        static_cast<T *>(P.Tout)[ic] = p * (rc2 * t * t) * cst<T>(P).inv_R;  // T = p/(rho R)
+    if (MODEL == JXF_SPM && P.viscous) static_cast<T *>(P.Tout)[ic] = (p * ir) * cst<T>(P).inv_R;  // T = p/(rho R)
     if constexpr (MODEL == JXF_DIM)
         if (P.thinc) (static_cast<T *>(P.G) + NDIM * nc)[ic] = thinc_psi(Wn[V::IA]);
+    s_out = T(0);
+    rho_out = rho;
+    bad = false;
+    if (!epi) return;
+    const T cs = rc2 * rsq(rho * rc2);
     T s = T(0);
 #pragma unroll
     for (int d = 0; d < NDIM; ++d) s += (fabs(Wn[V::NP + d]) + cs) * cst<T>(P).inv_dx[d];
     s_out = s;
-    rho_out = rho;
     bool ok = (rho > T(0)) && (rc2 > T(0)) && isfinite(rho) && isfinite(p) && (s == s);
 #pragma unroll
     for (int k = 0; k < V::NP; ++k) ok = ok && (U[k] > T(0));
@@ -2587,7 +2672,7 @@ __device__ __forceinline__ void finish_cell(const Dev &P, long long i, const T *
 // admissibility for the epilogue.  Shared by the single-grid and batched
 // updates.
 template <typename T, int MODEL, int NDIM>
-__device__ __forceinline__ void update_cell(const Dev &P, T cdt, long long i, int mode, T *U,
+__device__ __forceinline__ void update_cell(const Dev &P, T cdt, long long i, int mode, int epi, T *U,
                                             T &smax, T &rmin, bool &bad) {
     using V = Vars<MODEL, NDIM>;
     constexpr int NV = V::NV;
@@ -2646,7 +2731,7 @@ __device__ __forceinline__ void update_cell(const Dev &P, T cdt, long long i, in
         U[v] = first ? us[v] + cdt * R[v] : ca * un[v] + cb * us[v] + cdt * R[v];
         (Uo + v * nc)[ic] = U[v];
     }
-    finish_cell<T, MODEL, NDIM>(P, i, U, smax, rmin, bad);
+    finish_cell<T, MODEL, NDIM>(P, i, U, epi, smax, rmin, bad);
 }
 
 // c dt of the stage in the storage type, computed once per block.
@@ -2670,7 +2755,7 @@ __global__ void __launch_bounds__(kCellThreads, CellMinBlocks<T>::value)
     bool bad = false;
 #pragma unroll
     for (int v = 0; v < NV; ++v) U[v] = T(0);
-    if (i < P.ncell) update_cell<T, MODEL, NDIM>(P, cdt, i, mode, U, smax, rmin, bad);
+    if (i < P.ncell) update_cell<T, MODEL, NDIM>(P, cdt, i, mode, epi, U, smax, rmin, bad);
     if (mode == 1 && epi)
         block_partials<T, NV>(P, smax, rmin, bad, U, P.part + (size_t)blockIdx.x * (3 + MAXV));
 }
@@ -2776,7 +2861,7 @@ __global__ void __launch_bounds__(kFluxThreads, FusedMinBlocks<T, RSV>::value)
             }
             T s1, r1;
             bool b1;
-            finish_cell<T, MODEL, NDIM>(P, ic, U, s1, r1, b1);
+            finish_cell<T, MODEL, NDIM>(P, ic, U, epi, s1, r1, b1);
             if (epi) {
                 smax = tmax(smax, s1);
                 rmin = tmin(rmin, r1);
@@ -2834,11 +2919,11 @@ __global__ void __launch_bounds__(kFluxThreads, FusedMinBlocks<T, RSV>::value)
 // Primitives (+ temperature) of a conservative state, with the reduction
 // epilogue (used after the state is set).
 template <typename T, int MODEL, int NDIM>
-__device__ __forceinline__ void prim_cell(const Dev &P, long long i, T *U, T &smax, T &rmin, bool &bad) {
+__device__ __forceinline__ void prim_cell(const Dev &P, long long i, int epi, T *U, T &smax, T &rmin, bool &bad) {
     const T *Us = static_cast<const T *>(P.Us);
 #pragma unroll
     for (int v = 0; v < Vars<MODEL, NDIM>::NV; ++v) U[v] = Us[v * P.vstride + i];
-    finish_cell<T, MODEL, NDIM>(P, i, U, smax, rmin, bad);
+    finish_cell<T, MODEL, NDIM>(P, i, U, epi, smax, rmin, bad);
 }
 
 template <typename T, int MODEL, int NDIM>
@@ -2850,7 +2935,7 @@ __global__ void __launch_bounds__(kCellThreads) k_prim(const Dev P, const int ep
     bool bad = false;
 #pragma unroll
     for (int v = 0; v < NV; ++v) U[v] = T(0);
-    if (i < P.ncell) prim_cell<T, MODEL, NDIM>(P, i, U, smax, rmin, bad);
+    if (i < P.ncell) prim_cell<T, MODEL, NDIM>(P, i, epi, U, smax, rmin, bad);
     if (epi) block_partials<T, NV>(P, smax, rmin, bad, U, P.part + (size_t)blockIdx.x * (3 + MAXV));
 }
 
