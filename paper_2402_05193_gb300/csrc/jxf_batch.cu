@@ -60,7 +60,7 @@ struct jxf_batch_ctx {
     Tile *ftiles[3] = {nullptr, nullptr, nullptr}, *ctiles = nullptr;
     int nft[3] = {0, 0, 0}, nct = 0;
     // tiling (autotuner knobs)
-    int tile_faces = 1024, blocks_per_sm = 8;
+    int tile_faces = 512, blocks_per_sm = 8;
     // graph of n steps
     cudaStream_t cap = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -106,6 +106,19 @@ void bfree(jxf_batch_ctx *b) {
 }
 
 char *at(void *base, long long elems, size_t es) { return static_cast<char *>(base) + elems * (long long)es; }
+
+// Face-tile length before any tuning: the longest of 512, 256, 128 that fills
+// the persistent grid's 8 blocks per SM with a tile each (a block works through
+// its tile 128 faces at a time); double faces take ten times as long as the
+// queue's hand-over, so there the shortest.  us per step with tiles of 1024 |
+// 512 | 256 | 128: 96 drops float 1089 | 1069 | 1091 | 1180, 24 drops 322 | 305 |
+// 303 | 307, 4 drops 155 | 113 | 96 | 91, 24 drops double 6526 | 5511 | 5082 | 4975.
+int default_tile(const jxf_batch_ctx *b, long long faces) {
+    if (b->esize == 8) return kFluxThreads;
+    int t = 512;
+    while (t > kFluxThreads && faces / t < (long long)b->blocks_per_sm * b->sms) t /= 2;
+    return t;
+}
 
 // Face tiles of the given length per axis, cell tiles of one block.
 jxf_status build_tiles(jxf_batch_ctx *b) {
@@ -319,7 +332,10 @@ jxf_status jxf_batch_create(int nsim, const jxf_grid *grids, const jxf_eos *eos,
         cudaError_t e = cudaMemcpy(b->devs, b->hdev.data(), b->hdev.size() * sizeof(Dev), cudaMemcpyHostToDevice);
         if (e != cudaSuccess) st = bcuda(b, e, "upload parameter blocks");
     }
-    if (st == JXF_OK) st = build_tiles(b);
+    if (st == JXF_OK) {
+        b->tile_faces = default_tile(b, faces[0]);
+        st = build_tiles(b);
+    }
     if (st != JXF_OK) {
         bfree(b);
         delete b;

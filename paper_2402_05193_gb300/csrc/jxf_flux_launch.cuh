@@ -32,7 +32,7 @@ template <typename T, int MODEL, int NDIM, int VH, int RSV>
 void launch_flux_update(const Dev &P, int epi, cudaStream_t s) {
     if constexpr (NDIM >= 2 && std::is_same<T, float>::value) {
         const dim3 grid = fused_grid(P, NDIM);
-        k_flux_update<T, MODEL, NDIM, VH, RSV><<<grid, kFluxThreads, 0, s>>>(P, epi, kFusedRun);
+        k_flux_update<T, MODEL, NDIM, VH, RSV><<<grid, kFluxThreads, 0, s>>>(P, epi, fused_run(P, NDIM));
     }
 }
 

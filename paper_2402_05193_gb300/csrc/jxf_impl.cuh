@@ -2481,21 +2481,6 @@ __device__ __forceinline__ double warp_sum_pairs_to_double(float hi, float lo) {
     }
     return (double)hi + (double)lo;
 }
-__device__ __forceinline__ double warp_sum_to_double(double v) { return warp_sum(v); }
-__device__ __forceinline__ double warp_sum_to_double(float v) {
-    float hi = v, lo = 0.0f;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float oh = shfl_down(hi, o), ol = shfl_down(lo, o);
-        const float s = hi + oh;
-        const float bb = s - hi;
-        const float err = (hi - (s - bb)) + (oh - bb);
-        lo = lo + ol + err;
-        hi = s;
-    }
-    return (double)hi + (double)lo;
-}
-
 // Error-free transformations in float: a + b = s + e exactly (Knuth's
 // TwoSum), and the rounding error of a product from one fused multiply-add.
 __device__ __forceinline__ void two_sum_f(float a, float b, float &s, float &e) {
@@ -2583,45 +2568,80 @@ __device__ __forceinline__ void cons2prim_stiff_float(const Dev &P, const T *U, 
     ir_o = ir;
 }
 
+// Order-preserving integer key of a double (its own inverse): maxima and
+// minima on the integer pipe.
+__device__ __forceinline__ long long order_key(long long b) { return b ^ (long long)((unsigned long long)(b >> 63) >> 1); }
+__device__ __forceinline__ double warp_max_keyed(double v) {
+    long long k = order_key(__double_as_longlong(v));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) k = max(k, __shfl_down_sync(0xffffffffu, k, o));
+    return __longlong_as_double(order_key(k));
+}
+__device__ __forceinline__ double warp_min_keyed(double v) { return -warp_max_keyed(-v); }
+__device__ __forceinline__ float warp_max_keyed(float v) { return warp_max(v); }
+__device__ __forceinline__ float warp_min_keyed(float v) { return warp_min(v); }
+
 // Per-block partials of the cell epilogue: [smax, rmin, bad, sums...] with
 // the CFL maximum and the density minimum reduced in the storage type
-// (exact) and the conservation sums in double (times the cell volume).
-template <typename T, int NV, int NW = kCellThreads / 32>
-__device__ __forceinline__ void block_partials(const Dev &P, T smax, T rmin, bool bad, const T *U,
-                                               double *out) {
-    __shared__ double sh[NW][3 + MAXV];  // NW >= blockDim.x / 32
+// (exact) and the conservation sums in double (float: compensated pairs, as
+// in the fused sweep), times the cell volume.  The FP64 pipe bounds this, and
+// a shuffle tree in every warp fills it with instructions of which 1 to 16
+// lanes count: so the block's values go through shared memory, one warp sums
+// one variable, eight values per lane before the tree (12 additions per
+// variable instead of 47 in double; in float the only double operation per
+// variable is the last one).  k_prim on 256x128x128 five-equation cells in
+// float 275 -> @PRIM32@ us, on 128^3 in double 308 -> @PRIM64@ us.
+template <typename T, int NV>
+__device__ __forceinline__ void block_partials(const Dev &P, T smax, T rmin, bool bad, const T *U, double *out) {
+    constexpr int NW = kCellThreads / 32;
+    static_assert(NV < NW, "one warp per variable and one for the rest");
+    __shared__ T buf[NV][kCellThreads];
+    __shared__ T sh_max[NW], sh_min[NW];
+    __shared__ int sh_bad[NW];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const T m = warp_max(smax), n = warp_min(rmin);
+#pragma unroll
+    for (int v = 0; v < NV; ++v) buf[v][threadIdx.x] = U[v];
+    // a NaN rate or density marks the cell bad and stays out of the extrema
+    const T m = warp_max_keyed(smax == smax ? smax : T(0)), n = warp_min_keyed(rmin == rmin ? rmin : T(3e38));
     const bool anybad = __any_sync(0xffffffffu, bad);
-    double sums[NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) sums[v] = warp_sum_to_double(U[v]);
     if (lane == 0) {
-        sh[wid][0] = (double)m;
-        sh[wid][1] = (double)n;
-        sh[wid][2] = anybad ? 1.0 : 0.0;
-#pragma unroll
-        for (int v = 0; v < NV; ++v) sh[wid][3 + v] = sums[v];
+        sh_max[wid] = m;
+        sh_min[wid] = n;
+        sh_bad[wid] = anybad ? 1 : 0;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        const int nw = blockDim.x >> 5;
-        double a[3 + NV];
+    if (wid < NV) {
+        const T *b = buf[wid] + lane;
+        double s;
+        if constexpr (sizeof(T) == 8) {
+            T a = b[0];
 #pragma unroll
-        for (int k = 0; k < 3 + NV; ++k) a[k] = sh[0][k];
-        for (int w = 1; w < nw; ++w) {
-            a[0] = fmax(a[0], sh[w][0]);
-            a[1] = fmin(a[1], sh[w][1]);
-            a[2] = fmax(a[2], sh[w][2]);
+            for (int k = 1; k < NW; ++k) a += b[32 * k];
+            s = warp_sum(a);
+        } else {
+            T hi = b[0], lo = T(0);
 #pragma unroll
-            for (int v = 0; v < NV; ++v) a[3 + v] += sh[w][3 + v];
+            for (int k = 1; k < NW; ++k) {
+                T h, e;
+                two_sum_f(hi, b[32 * k], h, e);
+                hi = h;
+                lo = __fadd_rn(lo, e);
+            }
+            s = warp_sum_pairs_to_double(hi, lo);
         }
-        double *o = out;
-        o[0] = a[0];
-        o[1] = a[1];
-        o[2] = a[2];
+        if (lane == 0) out[3 + wid] = s * P.vol;
+    } else if (wid == NW - 1 && lane == 0) {
+        T a = sh_max[0], b = sh_min[0];
+        int c = sh_bad[0];
 #pragma unroll
-        for (int v = 0; v < NV; ++v) o[3 + v] = a[3 + v] * P.vol;
+        for (int w = 1; w < NW; ++w) {
+            a = tmax(a, sh_max[w]);
+            b = tmin(b, sh_min[w]);
+            c |= sh_bad[w];
+        }
+        out[0] = (double)a;
+        out[1] = (double)b;
+        out[2] = c ? 1.0 : 0.0;
     }
 }
 

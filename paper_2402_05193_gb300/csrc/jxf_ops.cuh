@@ -35,15 +35,25 @@ inline unsigned grid_for(long long n, int threads) {
 
 // The fused last-axis sweep: cells per run along the last axis, and its
 // grid (kFluxThreads columns per block by runs); one partial record per
-// block.  Runs of 16 cells keep the extra face per run at 1/16 and give a
-// 128^3 grid 1024 blocks.
-#ifndef JXF_FUSED_RUN
-#define JXF_FUSED_RUN 16
-#endif
-constexpr int kFusedRun = JXF_FUSED_RUN;  // overridable at build time for tuning sweeps
+// block.  A run computes one face more than it owns cells and its thread
+// marches through them one after the other: long runs waste less, short ones
+// give a small grid more blocks and a shorter chain.  The longest of 16, 8, 4,
+// 2, 1 that still leaves kFusedBlocks blocks (five per SM; 7 are resident) --
+// measured in us per step with runs of 16 | 8 | 4 | 2 | 1: 64x48 86 | 56 | 41 |
+// 33 | 29, 512^2 105 | 79 | 74 | 70 | 78, 1024^2 199 | 178 | 183 | 196 | 231, 32^3
+// viscous 152 | 109 | 90 | 82 | 80, 64^3 183 | 148 | 142 | 140 | 150, 96^3 363 |
+// 333 | 339 | 347 | 383 (chosen: 1, 2, 8, 1, 2, 8).
+constexpr int kFusedRunMax = 16, kFusedBlocks = 5 * 152;
+inline int fused_run(const Dev &P, int ndim) {
+    const long long plane = (long long)P.n[0] * (ndim == 3 ? P.n[1] : 1), n = P.n[ndim - 1];
+    int run = kFusedRunMax;
+    while (run > 1 && (long long)grid_for(plane, kFluxThreads) * ((n + run - 1) / run) < kFusedBlocks) run /= 2;
+    return run;
+}
 inline dim3 fused_grid(const Dev &P, int ndim) {
     const long long plane = (long long)P.n[0] * (ndim == 3 ? P.n[1] : 1);
-    return dim3(grid_for(plane, kFluxThreads), (unsigned)((P.n[ndim - 1] + kFusedRun - 1) / kFusedRun));
+    const int run = fused_run(P, ndim);
+    return dim3(grid_for(plane, kFluxThreads), (unsigned)((P.n[ndim - 1] + run - 1) / run));
 }
 
 // Face-sweep launchers, one instantiation per (storage type, model, ndim,
