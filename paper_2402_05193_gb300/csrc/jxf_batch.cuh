@@ -70,10 +70,9 @@ __global__ void __launch_bounds__(kFluxThreads, SweepMinBlocks<T, RSV>::value)
         const long long nface = (long long)m[0] * m[1] * m[2];
         const long long end = tl.start + tl.count;
         for (long long b = tl.start; b < end; b += blockDim.x) {
-            const long long g = b + threadIdx.x;
-            bool il = false, fl = false;
-            if (g < end) flux_face<T, MODEL, NDIM, d, VH, RSV>(P, dt, g, m, nface, il, fl);
-            if (P.limiter) count_limited(P, il, fl);
+            const int n = end - b < blockDim.x ? (int)(end - b) : (int)blockDim.x;
+            flux_block<T, MODEL, NDIM, d, VH, RSV, false>(P, dt, b, n, m, true, AllFaces{},
+                                                   FaceArrays<T, MODEL, NDIM, d>{P, nface});
         }
     }
 }

@@ -145,6 +145,7 @@ struct Dev {
     int weno_z;  // 0: Jiang-Shu weights, 1: WENO5-Z weights
     int teno;    // 1: TENO6-A instead of WENO5
     int viscous, limiter;
+    int split;   // double WENO5: resolved faces take the split correction (see kSplitFaces)
     int visc_half;  // viscous stencils: points per side (1, 2, 3 for order 2, 4, 6)
     int thinc;   // THINC volume-fraction reconstruction (five-equation model)
     double eps_rho, eps_rhoc2, eps_alpha, weno_eps;
@@ -877,11 +878,16 @@ __device__ __forceinline__ void recon_face(const T (&x)[6], T eps4, T &vl, T &vr
 // above; there the correction form would lose digits next to a jump (the
 // middle candidate's share of the jump cancels).  The choice is made per face
 // from its own stencil, so it does not depend on how faces are grouped into
-// warps.  One-dimensional grids keep the double formula for every face: they
-// are latency-bound, and a warp with a shock in it would pay for both
-// (200-cell tube: 70 against 73 us a step).
-// FP64 instructions of a 3-D viscous face: 620 -> 155; 128^3 Taylor-Green
-// step 24.8 -> 8.5 ms (sweeps 2.49 -> 0.74 ms each); right-hand sides against
+// warps.
+// Small grids (Dev::split = 0: no axis with more faces than one warp for each
+// of the 4 x 152 FP64 pipes, and all 1-D ones) keep the double formula for
+// every face: they are bound by the latency of one warp, and a warp with
+// faces of both kinds pays for both.  us per step, all double | by face: 128^2
+// shock-bubble 231 | 257, 24^3 waves 244 | 320, 200-cell tube 70 | 73.  With the
+// second warp per pipe the double formula takes twice as long: 160^2 bubble
+// 405 | 298, 160^2 waves 254 | 85, 40^3 815 | 295.
+// FP64 instructions of a 3-D viscous face: 620 -> 117; 128^3 Taylor-Green
+// step 24.8 -> 7.4 ms (sweeps 2.49 -> 0.60 ms each); right-hand sides against
 // float64 references are as close as before (1.1e-14 -> 0.9e-14 on smooth
 // 3-D fields).  Three blocks of 128 an SM (168 registers) let the integer and
 // FP32 work of one warp run beside the FP64 work of the others: 8.75 ms
@@ -1006,6 +1012,7 @@ __device__ __forceinline__ double widen(float x) {
     return __hiloint2double((int)((((b & 0x7FFFFFFFu) >> 3) + 0x38000000u) | (b & 0x80000000u)), (int)(b << 29));
 }
 
+constexpr long long kSplitFaces = 4 * 152 * 32 + 1;
 constexpr float kSplitD = 1.f / 16.f;   // bound of |D| over the variable's scale
 constexpr float kSplitT = 1.f / 128.f;  // bound of |T|
 
@@ -1046,45 +1053,24 @@ template <int MODEL, int NDIM> struct Frozen {
     }
 };
 
-// Face states of a double WENO5 face by the split correction; false (nothing
-// written) where the stencil is not resolved enough for it, or its scales
-// leave the range the float pairs are normal numbers in.
-template <int MODEL, int NDIM, int d>
-__device__ __forceinline__ bool reconstruct_split(const Dev &P, const double (&S)[6][MAXV], double *WL, double *WR) {
+// Whether a face takes the split correction: largest |D| and |T| of each
+// variable (dm, tm), the state w2 of cell 2 and the stencil's largest high
+// word `top` against the bounds; scales in the range in which the float pairs
+// are normal numbers.
+template <int MODEL, int NDIM>
+__device__ __forceinline__ bool split_bounds(const Dev &P, const float (&dm)[Vars<MODEL, NDIM>::NV],
+                                             const float (&tm)[Vars<MODEL, NDIM>::NV],
+                                             const float (&w2)[Vars<MODEL, NDIM>::NV], unsigned top) {
     using V = Vars<MODEL, NDIM>;
-    constexpr int NV = V::NV, NP = V::NP, IE = V::IE, in = NP + d;
-    const bool z = P.weno_z != 0;
+    constexpr int NV = V::NV, NP = V::NP, IE = V::IE;
     const Cst<float> &C = P.k32;
     const bool chr = P.recon != JXF_WENO5JS_COMP;
-    float Dh[5][NV], Dl[5][NV];
-    float dm[NV], tm[NV];
-    unsigned top = 0;  // largest exponent word of the stencil
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-#pragma unroll
-        for (int k = 0; k < 6; ++k) top = max(top, (unsigned)__double2hiint(S[k][v]) & 0x7FFFFFFFu);
-#pragma unroll
-        for (int k = 0; k < 5; ++k) split_double(S[k + 1][v] - S[k][v], Dh[k][v], Dl[k][v]);
-        dm[v] = fmaxf(fmaxf(fmaxf(fabsf(Dh[0][v]), fabsf(Dh[1][v])), fmaxf(fabsf(Dh[2][v]), fabsf(Dh[3][v]))),
-                      fabsf(Dh[4][v]));
-        float t = 0.f;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) t = fmaxf(t, fabsf((Dh[k][v] - Dh[k + 1][v]) + (Dh[k + 2][v] - Dh[k + 1][v])));
-        tm[v] = t;
-    }
-    // frozen state: mean of the face's two cells, S2 + D2/2, in pairs
-    float wh[NV], wl[NV];
-    float rho = 0.f;
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-        if (v < NP || v == IE || v == V::IA) split_double(S[2][v], wh[v], wl[v]);
-        if (v < NP) rho += wh[v];
-    }
-    float rc2;
-    if (MODEL == JXF_SPM) rc2 = C.gamma0 * (wh[IE] + C.pinf0);
+    float rho = w2[0], rc2;
+    if (NP == 2) rho += w2[NP - 1];
+    if (MODEL == JXF_SPM) rc2 = C.gamma0 * (w2[IE] + C.pinf0);
     else {
-        const float a1 = wh[V::IA >= 0 ? V::IA : 0];
-        rc2 = wh[IE] + (wh[IE] + (C.B2h + a1 * C.dBh)) * rcp(C.A2h + a1 * C.dAh);
+        const float a1 = w2[V::IA >= 0 ? V::IA : 0];
+        rc2 = w2[IE] + (w2[IE] + (C.B2h + a1 * C.dBh)) * rcp(C.A2h + a1 * C.dAh);
     }
     const float c = rc2 * rsq(rho * rc2);
     bool ok = top < 0x47600000u && rho > 1.5e-5f && rho < 1e10f && rc2 > 1.5e-5f && rc2 < 1e18f && c > 1.5e-5f;
@@ -1097,7 +1083,69 @@ __device__ __forceinline__ bool reconstruct_split(const Dev &P, const double (&S
         if (!chr) ok = ok && dm[v] * dm[v] <= qlim;
         else ok = ok && (v == IE ? 0.01f : (kSplitD * kSplitD * 4.f) * sc * sc) <= qlim;
     }
-    if (!ok) return false;
+    return ok;
+}
+__device__ __forceinline__ void split_sizes(float D0, float D1, float D2, float D3, float D4, float &dm, float &tm) {
+    dm = fmaxf(fmaxf(fmaxf(fabsf(D0), fabsf(D1)), fmaxf(fabsf(D2), fabsf(D3))), fabsf(D4));
+    tm = fmaxf(fmaxf(fabsf((D0 - D1) + (D2 - D1)), fabsf((D1 - D2) + (D3 - D2))), fabsf((D2 - D3) + (D4 - D3)));
+}
+
+// The same from the high words hi(j, v) of the stencil's doubles alone
+// (values truncated to 20 bits: enough for bounds that leave a factor of 8 and
+// more to what matters), without FP64 work.
+template <int MODEL, int NDIM, int d, class Hi>
+__device__ __forceinline__ bool face_resolved(const Dev &P, Hi hi) {
+    constexpr int NV = Vars<MODEL, NDIM>::NV;
+    float dm[NV], tm[NV], w2[NV];
+    unsigned top = 0;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+        float x[6];
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+            const unsigned h = hi(j, v), a = h & 0x7FFFFFFFu;
+            top = max(top, a);
+            // the exponent's low 8 bits rebiased by 896 = flip of their top bit
+            const unsigned b = (((h << 3) ^ 0x40000000u) & 0x7FFFFFFFu) | (h & 0x80000000u);
+            x[j] = a < 0x38100000u ? 0.f : __uint_as_float(b);
+        }
+        w2[v] = x[2];
+        split_sizes(x[1] - x[0], x[2] - x[1], x[3] - x[2], x[4] - x[3], x[5] - x[4], dm[v], tm[v]);
+    }
+    return split_bounds<MODEL, NDIM>(P, dm, tm, w2, top);
+}
+
+// Face states of a double WENO5 face by the split correction; TRY: if the
+// face is resolved, else false and nothing written.
+template <int MODEL, int NDIM, int d, bool TRY>
+__device__ __forceinline__ bool reconstruct_split(const Dev &P, const double (&S)[6][MAXV], double *WL, double *WR) {
+    using V = Vars<MODEL, NDIM>;
+    constexpr int NV = V::NV, NP = V::NP, IE = V::IE, in = NP + d;
+    const bool z = P.weno_z != 0;
+    const Cst<float> &C = P.k32;
+    const bool chr = P.recon != JXF_WENO5JS_COMP;
+    float Dh[5][NV], Dl[5][NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+#pragma unroll
+        for (int k = 0; k < 5; ++k) split_double(S[k + 1][v] - S[k][v], Dh[k][v], Dl[k][v]);
+    }
+    // frozen state: mean of the face's two cells, S2 + D2/2, in pairs
+    float wh[NV], wl[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v)
+        if (v < NP || v == IE || v == V::IA) split_double(S[2][v], wh[v], wl[v]);
+    if constexpr (TRY) {
+        float dm[NV], tm[NV];
+        unsigned top = 0;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+#pragma unroll
+            for (int j = 0; j < 6; ++j) top = max(top, (unsigned)__double2hiint(S[j][v]) & 0x7FFFFFFFu);
+            split_sizes(Dh[0][v], Dh[1][v], Dh[2][v], Dh[3][v], Dh[4][v], dm[v], tm[v]);
+        }
+        if (!split_bounds<MODEL, NDIM>(P, dm, tm, wh, top)) return false;
+    }
 
     auto pair = [&](int k, int v) {
         return d2{mk2(Dh[k][v], Dh[4 - k][v]), mk2(Dl[k][v], Dl[4 - k][v])};
@@ -1373,14 +1421,21 @@ __device__ __forceinline__ void reconstruct_w(const Dev &P, const T (&S)[6][MAXV
 // RSV: the kernel variant's scheme family -- 0: WENO5 (Jiang-Shu or Z
 // weights, chosen per face from P.weno_z), 2: TENO6-A (its own kernels, so
 // that its registers do not weigh on the WENO5 sweeps).
-// Returns how a double face was reconstructed.
-enum { FACE_FULL = 0, FACE_SPLIT = 1, FACE_CENTRAL = 2 };
-template <typename T, int MODEL, int NDIM, int d, int RSV>
+// HOW a double face is reconstructed: all in double, with the split
+// correction (the caller knows it is resolved), or TRY: TENO6-A by the central
+// value if all candidates are kept for certain, WENO5 split if resolved.
+// Returns how it was, FACE_NONE if a TENO6-A face tried is not certain.
+enum { FACE_NONE = -1, FACE_FULL = 0, FACE_SPLIT = 1, FACE_CENTRAL = 2, FACE_TRY = 3 };
+template <typename T, int MODEL, int NDIM, int d, int RSV, int HOW>
 __device__ __forceinline__ int reconstruct(const Dev &P, const T (&S)[6][MAXV], T *WL, T *WR) {
-    if constexpr (std::is_same<T, double>::value && RSV == 0 && NDIM > 1)
-        if (reconstruct_split<MODEL, NDIM, d>(P, S, WL, WR)) return FACE_SPLIT;
-    if constexpr (std::is_same<T, double>::value && RSV == 2)
-        if (reconstruct_central<MODEL, NDIM, d>(P, S, WL, WR)) return FACE_CENTRAL;
+    if constexpr (std::is_same<T, double>::value && HOW == FACE_SPLIT) {
+        reconstruct_split<MODEL, NDIM, d, false>(P, S, WL, WR);
+        return FACE_SPLIT;
+    }
+    if constexpr (std::is_same<T, double>::value && HOW == FACE_TRY && RSV == 2)
+        return reconstruct_central<MODEL, NDIM, d>(P, S, WL, WR) ? FACE_CENTRAL : FACE_NONE;
+    if constexpr (std::is_same<T, double>::value && HOW == FACE_TRY && RSV != 2 && NDIM > 1)
+        if (P.split && reconstruct_split<MODEL, NDIM, d, true>(P, S, WL, WR)) return FACE_SPLIT;
     if constexpr (RSV == 2) reconstruct_w<T, MODEL, NDIM, d, 2>(P, S, WL, WR);
     else if (P.weno_z) reconstruct_w<T, MODEL, NDIM, d, 1>(P, S, WL, WR);
     else reconstruct_w<T, MODEL, NDIM, d, 0>(P, S, WL, WR);
@@ -2166,24 +2221,20 @@ template <typename T, int MODEL, int NDIM, int d, bool MIR> struct GlobalStencil
 // gather, reconstruction, interpolation limiter, HLLC, flux limiter, viscous
 // flux; returns F (and u_hllc).  Shared by the single-grid sweep, the fused
 // last-axis sweep and the batched persistent sweep.
-// VH: points per side of the viscous stencils (0: no viscous flux).
-template <typename T, int MODEL, int NDIM, int d, int VH, int RSV, typename Src>
-__device__ __forceinline__ void flux_face_eval(const Dev &P, double dt, const int (&c)[3], const Src &src, bool count,
+// VH: points per side of the viscous stencils (0: no viscous flux); HOW: how
+// a double face is reconstructed (false: a tried TENO6-A face that needs the
+// full evaluation, nothing written).
+template <typename T, int MODEL, int NDIM, int d, int VH, int RSV, int HOW, typename Src>
+__device__ __forceinline__ bool flux_face_eval(const Dev &P, double dt, const int (&c)[3], const Src &src, bool count,
                                                T (&F)[MAXV], T &uh, bool &il_hit, bool &fl_hit);
 
-// The flux F (= F^c - F^d) and upwinded velocity uh of the face of axis d at
-// face coordinates c (face c[d] lies between cells c[d]-1 and c[d]).
-// count = false: the face is computed a second time (by a block that shares
-// it) and stays out of the limiter counters.
-template <typename T, int MODEL, int NDIM, int d, int VH, int RSV>
-__device__ __forceinline__ void flux_face_at(const Dev &P, double dt, const int (&c)[3], bool count,
-                                             T (&F)[MAXV], T &uh, bool &il_hit, bool &fl_hit) {
-    // face c[d] lies between cells c[d]-1 (i) and c[d] (i+1).  Stencil
-    // cells i-2..i+3 differ only along d: map that coordinate through
-    // the boundary conditions once per cell (bit j of mir: mirrored).
+// Cell indices of the stencil of the face of axis d at face coordinates c
+// (face c[d] lies between cells c[d]-1 (i) and c[d] (i+1); stencil cells
+// i-2..i+3 differ only along d: that coordinate is mapped through the boundary
+// conditions once per cell); bit j of the result: cell j is mirrored.
+template <int d> __device__ __forceinline__ unsigned stencil_cells(const Dev &P, const int (&c)[3], int (&idx)[6]) {
     const int sd = d == 0 ? 1 : (d == 1 ? P.n[0] : P.n[0] * P.n[1]);
     const int base = ((c[2] * P.n[1] + c[1]) * P.n[0] + c[0]) - c[d] * sd;
-    int idx[6];
     unsigned mir = 0;
     if (c[d] >= 3 && c[d] <= P.n[d] - 3) {  // whole stencil inside: no mapping
 #pragma unroll
@@ -2197,6 +2248,17 @@ __device__ __forceinline__ void flux_face_at(const Dev &P, double dt, const int 
             mir |= (unsigned)mj << j;
         }
     }
+    return mir;
+}
+
+// The flux F (= F^c - F^d) and upwinded velocity uh of the face of axis d at
+// face coordinates c.  count = false: the face is computed a second time (by
+// a block that shares it) and stays out of the limiter counters.
+template <typename T, int MODEL, int NDIM, int d, int VH, int RSV, int HOW>
+__device__ __forceinline__ bool flux_face_at(const Dev &P, double dt, const int (&c)[3], bool count,
+                                             T (&F)[MAXV], T &uh, bool &il_hit, bool &fl_hit) {
+    int idx[6];
+    const unsigned mir = stencil_cells<d>(P, c, idx);
     // Float sweeps across y or z: the stencil's mirror pattern is constant
     // along a row of x-faces (so over a warp when the row length is a
     // multiple of 32); faces without mirrored cells take a copy of the face
@@ -2204,34 +2266,26 @@ __device__ __forceinline__ void flux_face_at(const Dev &P, double dt, const int 
     if constexpr (d > 0 && std::is_same<T, float>::value) {
         if (mir == 0u) {
             const GlobalStencil<T, MODEL, NDIM, d, false> src{P, idx, 0u};
-            flux_face_eval<T, MODEL, NDIM, d, VH, RSV>(P, dt, c, src, count, F, uh, il_hit, fl_hit);
-            return;
+            return flux_face_eval<T, MODEL, NDIM, d, VH, RSV, HOW>(P, dt, c, src, count, F, uh, il_hit, fl_hit);
         }
     }
     const GlobalStencil<T, MODEL, NDIM, d, true> src{P, idx, mir};
-    flux_face_eval<T, MODEL, NDIM, d, VH, RSV>(P, dt, c, src, count, F, uh, il_hit, fl_hit);
+    return flux_face_eval<T, MODEL, NDIM, d, VH, RSV, HOW>(P, dt, c, src, count, F, uh, il_hit, fl_hit);
 }
 
-// Face g of axis d (x-fastest index over the faces of axis d): its flux into
-// the face arrays.
-template <typename T, int MODEL, int NDIM, int d, int VH, int RSV>
-__device__ __forceinline__ void flux_face(const Dev &P, double dt, long long g, const int (&m)[3],
-                                          long long nface, bool &il_hit, bool &fl_hit) {
+// Coordinates of face g of axis d (x-fastest index over the faces of axis d,
+// extents m).
+template <int d> __device__ __forceinline__ void face_coords(const Dev &P, long long g, const int (&m)[3], int (&c)[3]) {
     const unsigned gu = (unsigned)g;
     const unsigned q0 = P.fd_face[d][0].div(gu);
     const unsigned q1 = P.fd_face[d][1].div(q0);
-    const int c[3] = {(int)(gu - q0 * (unsigned)m[0]), (int)(q0 - q1 * (unsigned)m[1]), (int)q1};
-    T F[MAXV], uh;
-    flux_face_at<T, MODEL, NDIM, d, VH, RSV>(P, dt, c, true, F, uh, il_hit, fl_hit);
-    constexpr int NV = Vars<MODEL, NDIM>::NV;
-    T *Fo = static_cast<T *>(P.F[d]);
-#pragma unroll
-    for (int v = 0; v < NV; ++v) (Fo + v * nface)[(int)g] = F[v];  // g < 2^31 (checked at creation)
-    if (MODEL == JXF_DIM) static_cast<T *>(P.UH[d])[(int)g] = uh;
+    c[0] = (int)(gu - q0 * (unsigned)m[0]);
+    c[1] = (int)(q0 - q1 * (unsigned)m[1]);
+    c[2] = (int)q1;
 }
 
-template <typename T, int MODEL, int NDIM, int d, int VH, int RSV, typename Src>
-__device__ __forceinline__ void flux_face_eval(const Dev &P, double dt, const int (&c)[3], const Src &src, bool count,
+template <typename T, int MODEL, int NDIM, int d, int VH, int RSV, int HOW, typename Src>
+__device__ __forceinline__ bool flux_face_eval(const Dev &P, double dt, const int (&c)[3], const Src &src, bool count,
                                                T (&F)[MAXV], T &uh, bool &il_hit, bool &fl_hit) {
     using V = Vars<MODEL, NDIM>;
     constexpr int NV = V::NV;
@@ -2241,14 +2295,19 @@ __device__ __forceinline__ void flux_face_eval(const Dev &P, double dt, const in
 #pragma unroll
         for (int v = 0; v < NV; ++v) S[j][v] = src.w(j, v);
     }
+    T WL[MAXV], WR[MAXV];
+    int how = FACE_FULL;
+    if constexpr (HOW == FACE_TRY) {  // may not be this face's way: first
+        how = reconstruct<T, MODEL, NDIM, d, RSV, HOW>(P, S, WL, WR);
+        if (how == FACE_NONE) return false;
+    }
     // dissipative flux first, while the stencil's velocities are at hand
     T Fd[MAXV];
     if constexpr (MODEL == JXF_SPM && VH > 0) {
         if constexpr (std::is_same<T, double>::value) viscous_flux_double<NDIM, d, VH>(P, src, S, Fd);
         else viscous_flux<T, NDIM, d, VH>(P, src, S, Fd);
     }
-    T WL[MAXV], WR[MAXV];
-    int how = reconstruct<T, MODEL, NDIM, d, RSV>(P, S, WL, WR);
+    if constexpr (HOW != FACE_TRY) how = reconstruct<T, MODEL, NDIM, d, RSV, HOW>(P, S, WL, WR);
     if constexpr (MODEL == JXF_DIM) {
         if (P.thinc) {  // cell i's upper face value, cell i+1's lower face value
             constexpr int IA = V::IA;
@@ -2272,9 +2331,9 @@ __device__ __forceinline__ void flux_face_eval(const Dev &P, double dt, const in
 #pragma unroll 1
     for (int pass = 0;; ++pass) {
         bool done = false;
-        if constexpr (std::is_same<T, double>::value && RSV == 0 && NDIM > 1)
+        if constexpr (std::is_same<T, double>::value && RSV == 0 && NDIM > 1 && HOW != FACE_FULL)
             if (how == FACE_SPLIT && pass == 0) done = hllc_split<MODEL, NDIM, d>(P, WL, WR, F, uh);
-        if constexpr (std::is_same<T, double>::value && RSV == 2)
+        if constexpr (std::is_same<T, double>::value && HOW == FACE_TRY && RSV == 2)
             if (how == FACE_CENTRAL && pass == 0) done = hllc_equal<MODEL, NDIM, d>(P, WL, F, uh);
         if (!done) hllc<T, MODEL, NDIM, d>(P, WL, WR, F, uh);
         if (pass > 0 || !P.limiter) break;
@@ -2294,6 +2353,7 @@ __device__ __forceinline__ void flux_face_eval(const Dev &P, double dt, const in
 #pragma unroll
         for (int v = 0; v < NV; ++v) F[v] -= Fd[v];
     }
+    return true;
 }
 
 // Limiter activity of a warp into the counters (all lanes must call).
@@ -2306,6 +2366,121 @@ __device__ __forceinline__ void count_limited(const Dev &P, bool il_hit, bool fl
     }
 }
 
+// Every face is to be evaluated / its flux goes to the face arrays.
+struct AllFaces {
+    __device__ __forceinline__ bool operator()(long long) const { return true; }
+};
+template <typename T, int MODEL, int NDIM, int d> struct FaceArrays {
+    const Dev &P;
+    long long nface;
+    __device__ __forceinline__ void operator()(long long g, const T *F, T uh) const {
+        constexpr int NV = Vars<MODEL, NDIM>::NV;
+        T *Fo = static_cast<T *>(P.F[d]);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) (Fo + v * nface)[(int)g] = F[v];  // g < 2^31 (checked at creation)
+        if (MODEL == JXF_DIM) static_cast<T *>(P.UH[d])[(int)g] = uh;
+    }
+};
+
+// Face g into put; false: a tried TENO6-A face needs the full evaluation.
+template <typename T, int MODEL, int NDIM, int d, int VH, int RSV, int HOW, class Put>
+__device__ __forceinline__ bool flux_one(const Dev &P, double dt, long long g, const int (&m)[3], bool count,
+                                         const Put &put, bool &il, bool &fl) {
+    int c[3];
+    face_coords<d>(P, g, m, c);
+    T F[MAXV], uh;
+    if (!flux_face_at<T, MODEL, NDIM, d, VH, RSV, HOW>(P, dt, c, count, F, uh, il, fl)) return false;
+    put(g, F, uh);
+    return true;
+}
+
+// Faces base .. base + n - 1 of axis d by one block (n <= kFluxThreads; every
+// thread calls): those that wet(g) wants, their fluxes to put(g, F, uh).
+//
+// Double faces come in two kinds, resolved ones (split correction, or TENO6-A
+// with all candidates kept) and the rest; a warp with both runs both codes, one
+// after the other.  TENO6-A, whose long evaluation takes ten times the short
+// one, runs the short one and gathers the block's faces it was not enough for
+// (67x58x45 between walls 1.05 -> 0.89 ms).  SORT (the level-set model, most of
+// whose faces are dry and whose interface is lined with unresolved ones): the
+// block sorts its faces beforehand, by integer and float work on the high
+// words, into two lists whose warps are each of one kind, the long ones
+// starting first and a fifth warpful going to the first warp that is done
+// (96^3 drop 10.1 -> 9.9 ms).  Sorting costs 7 % where nothing needs it
+// (128^3 Taylor-Green 7.4 -> 8.0 ms), so the other sweeps choose lane by lane.
+// How a face is evaluated depends on its own stencil only.
+template <typename T, int MODEL, int NDIM, int d, int VH, int RSV, bool SORT, class Wet, class Put>
+__device__ __forceinline__ void flux_block(const Dev &P, double dt, long long base, int n, const int (&m)[3],
+                                           bool count, const Wet &wet, const Put &put) {
+    const int tid = threadIdx.x, lane = tid & 31;
+    constexpr bool kGather = std::is_same<T, double>::value && RSV == 2;
+    constexpr bool kSort = std::is_same<T, double>::value && RSV != 2 && NDIM > 1 && SORT;
+    bool il = false, fl = false;
+    if constexpr (kGather || kSort) {
+        __shared__ unsigned char list[kFluxThreads];
+        __shared__ int cnt[2], next;
+        __syncthreads();  // the previous use of the lists is over
+        if (tid == 0) cnt[0] = cnt[1] = 0, next = kFluxThreads / 32;
+        __syncthreads();
+        // position of this lane's face among those counted in cnt[k]
+        auto place = [&](bool want, int k) {
+            const unsigned mask = __ballot_sync(0xffffffffu, want);
+            int b = 0;
+            if (mask && lane == 0) b = atomicAdd(&cnt[k], __popc(mask));
+            return __shfl_sync(0xffffffffu, b, 0) + __popc(mask & ((1u << lane) - 1u));
+        };
+        if constexpr (kGather) {
+            const bool left = tid < n && wet(base + tid) && !flux_one<T, MODEL, NDIM, d, VH, RSV, FACE_TRY>(P, dt, base + tid, m, count, put, il, fl);
+            if (P.limiter) count_limited(P, il, fl);
+            const int at = place(left, 0);
+            if (left) list[at] = (unsigned char)tid;
+            __syncthreads();
+            if ((tid & ~31) < cnt[0]) {  // warp-uniform
+                il = fl = false;
+                if (tid < cnt[0]) flux_one<T, MODEL, NDIM, d, VH, RSV, FACE_FULL>(P, dt, base + list[tid], m, count, put, il, fl);
+                if (P.limiter) count_limited(P, il, fl);
+            }
+        } else {
+            const bool in = tid < n && wet(base + tid);
+            bool res = false;
+            if (in && P.split) {
+                int c[3], idx[6];
+                face_coords<d>(P, base + tid, m, c);
+                const unsigned mir = stencil_cells<d>(P, c, idx);
+                const unsigned *W = static_cast<const unsigned *>(P.W);
+                constexpr int vn = Vars<MODEL, NDIM>::NP + d;
+                res = face_resolved<MODEL, NDIM, d>(P, [&](int j, int v) {
+                    const unsigned h = __ldg(W + 2 * (v * (size_t)P.vstride + idx[j]) + 1);
+                    return v == vn && ((mir >> j) & 1u) ? h ^ 0x80000000u : h;
+                });
+            }
+            const int af = place(in && !res, 0), ar = place(res, 1);
+            if (in) list[res ? ar : kFluxThreads - 1 - af] = (unsigned char)tid;
+            __syncthreads();
+            const int nf = (cnt[0] + 31) >> 5, nr = (cnt[1] + 31) >> 5;
+            for (int t = tid >> 5; t < nf + nr;) {
+                il = fl = false;
+                if (t < nf) {
+                    const int i = t * 32 + lane;
+                    if (i < cnt[0]) flux_one<T, MODEL, NDIM, d, VH, RSV, FACE_FULL>(P, dt, base + list[kFluxThreads - 1 - i], m, count, put, il, fl);
+                } else {
+                    const int i = (t - nf) * 32 + lane;
+                    if (i < cnt[1]) flux_one<T, MODEL, NDIM, d, VH, RSV, FACE_SPLIT>(P, dt, base + list[i], m, count, put, il, fl);
+                }
+                if (P.limiter) count_limited(P, il, fl);
+                if (lane == 0) t = atomicAdd(&next, 1);
+                t = __shfl_sync(0xffffffffu, t, 0);
+            }
+        }
+    } else {
+        if (tid < n && wet(base + tid)) {
+            if constexpr (std::is_same<T, double>::value && NDIM > 1) flux_one<T, MODEL, NDIM, d, VH, RSV, FACE_TRY>(P, dt, base + tid, m, count, put, il, fl);
+            else flux_one<T, MODEL, NDIM, d, VH, RSV, FACE_FULL>(P, dt, base + tid, m, count, put, il, fl);
+        }
+        if (P.limiter) count_limited(P, il, fl);
+    }
+}
+
 template <typename T, int MODEL, int NDIM, int d, int VH, int RSV>
 __global__ void __launch_bounds__(kFluxThreads, SweepMinBlocks<T, RSV>::value) k_flux(const Dev P) {
     double dt;
@@ -2313,10 +2488,9 @@ __global__ void __launch_bounds__(kFluxThreads, SweepMinBlocks<T, RSV>::value) k
     int m[3] = {P.n[0], P.n[1], P.n[2]};
     m[d] += 1;
     const long long nface = (long long)m[0] * m[1] * m[2];
-    const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    bool il_hit = false, fl_hit = false;
-    if (g < nface) flux_face<T, MODEL, NDIM, d, VH, RSV>(P, dt, g, m, nface, il_hit, fl_hit);
-    if (P.limiter) count_limited(P, il_hit, fl_hit);
+    const long long base = (long long)blockIdx.x * blockDim.x;
+    const int n = nface - base < blockDim.x ? (int)(nface - base) : (int)blockDim.x;
+    flux_block<T, MODEL, NDIM, d, VH, RSV, false>(P, dt, base, n, m, true, AllFaces{}, FaceArrays<T, MODEL, NDIM, d>{P, nface});
 }
 
 // -------------------------------------------------- block reductions -----
@@ -2435,7 +2609,7 @@ __global__ void __launch_bounds__(kFluxThreads, SweepMinBlocks<T, RSV>::value) k
             if (NDIM == 3) c[3 - d] = o;
             const TileStencil<T, MODEL, NDIM, d, VH, kTileX * NA> src{P, sm + ((f - d0) * kTileX + lane) * NA, c};
             T F[MAXV], uh;
-            flux_face_eval<T, MODEL, NDIM, d, VH, RSV>(P, dt, c, src, true, F, uh, il, fl);
+            flux_face_eval<T, MODEL, NDIM, d, VH, RSV, FACE_FULL>(P, dt, c, src, true, F, uh, il, fl);
             const int g = chk_face(P, ((long long)c[2] * m[1] + c[1]) * m[0] + c[0], nface);
 #pragma unroll
             for (int v = 0; v < NV; ++v) (Fo + v * nface)[g] = F[v];
@@ -2590,7 +2764,7 @@ __device__ __forceinline__ float warp_min_keyed(float v) { return warp_min(v); }
 // one variable, eight values per lane before the tree (12 additions per
 // variable instead of 47 in double; in float the only double operation per
 // variable is the last one).  k_prim on 256x128x128 five-equation cells in
-// float 275 -> @PRIM32@ us, on 128^3 in double 308 -> @PRIM64@ us.
+// float 275 -> 45 us, on 128^3 in double 308 -> 184 us.
 template <typename T, int NV>
 __device__ __forceinline__ void block_partials(const Dev &P, T smax, T rmin, bool bad, const T *U, double *out) {
     constexpr int NW = kCellThreads / 32;
@@ -2827,7 +3001,7 @@ __global__ void __launch_bounds__(kFluxThreads, FusedMinBlocks<T, RSV>::value)
         c[d] = f;
         T F[MAXV], uh = T(0);
         bool il = false, fl = false;
-        if (active) flux_face_at<T, MODEL, NDIM, d, VH, RSV>(P, dt, c, f < d1 || d1 == nd, F, uh, il, fl);
+        if (active) flux_face_at<T, MODEL, NDIM, d, VH, RSV, FACE_FULL>(P, dt, c, f < d1 || d1 == nd, F, uh, il, fl);
         if (P.limiter) count_limited(P, il, fl);
         if (active && f > d0) {  // cell f-1 between the faces Fm (below) and F (above)
             const int z = f - 1;

@@ -811,22 +811,21 @@ __global__ void __launch_bounds__(jxf::kFluxThreads, jxf::SweepMinBlocks<double,
     int m[3] = {P.n[0], P.n[1], P.n[2]};
     m[d] += 1;
     const long long nface = (long long)m[0] * m[1] * m[2];
-    const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= nface) return;
-    const double A = __ldg(apd + g);
-    if (phase == 1 ? !(A > 0.0) : !(A < 1.0)) {
+    const long long g = (long long)blockIdx.x * blockDim.x;
+    const auto wet = [&](long long f) {
+        const double A = __ldg(apd + f);
+        if (phase == 1 ? A > 0.0 : A < 1.0) return true;
 #pragma unroll
-        for (int v = 0; v < V::NV; ++v) F[v * nface + g] = 0.0;
-        return;
-    }
-    const unsigned gu = (unsigned)g;
-    const unsigned q0 = P.fd_face[d][0].div(gu), q1 = P.fd_face[d][1].div(q0);
-    const int c[3] = {(int)(gu - q0 * (unsigned)m[0]), (int)(q0 - q1 * (unsigned)m[1]), (int)q1};
-    double Fv[jxf::MAXV], uh;
-    bool il = false, fl = false;
-    jxf::flux_face_at<double, JXF_SPM, NDIM, d, 0, RSV>(P, 0.0, c, false, Fv, uh, il, fl);
+        for (int v = 0; v < V::NV; ++v) F[v * nface + f] = 0.0;
+        return false;
+    };
+    const auto put = [&](long long f, const double *Fv, double) {
 #pragma unroll
-    for (int v = 0; v < V::NV; ++v) F[v * nface + g] = Fv[v];
+        for (int v = 0; v < V::NV; ++v) F[v * nface + f] = Fv[v];
+    };
+    const long long left = nface - g;
+    jxf::flux_block<double, JXF_SPM, NDIM, d, 0, RSV, true>(P, 0.0, g, left < blockDim.x ? (int)left : (int)blockDim.x, m,
+                                                       false, wet, put);
 }
 
 // d(alpha U)/dt of phase 1 (phi > 0) or 2 in every cell: the face fluxes

@@ -119,6 +119,13 @@ inline void fill_dev(const jxf_grid *grid, const jxf_eos *eos, const jxf_scheme 
     P.thinc = scheme->thinc && eos->model == JXF_DIM ? 1 : 0;
     P.limiter = scheme->limiter ? 1 : 0;
     const bool f64 = scheme->precision == JXF_FP64;
+    // by the whole grid, also for a block of it: the blocks' faces are evaluated
+    // as the grid's
+    for (int d = 0; d < grid->ndim; ++d) {
+        long long nf = 1;
+        for (int e = 0; e < grid->ndim; ++e) nf *= grid->n[e] + (e == d ? 1 : 0);
+        if (grid->ndim > 1 && nf >= kSplitFaces) P.split = 1;
+    }
     P.eps_rho = scheme->eps_rho > 0.0 ? scheme->eps_rho : (f64 ? 1e-12 : 1e-10);
     P.eps_rhoc2 = scheme->eps_rhoc2 > 0.0 ? scheme->eps_rhoc2 : (f64 ? 1e-10 : 1e-8);
     P.eps_alpha = scheme->eps_alpha > 0.0 ? scheme->eps_alpha : (f64 ? 1e-12 : 1e-10);
