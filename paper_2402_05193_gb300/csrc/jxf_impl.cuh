@@ -1263,6 +1263,14 @@ __device__ __forceinline__ bool reconstruct_central(const Dev &P, const double (
     using V = Vars<MODEL, NDIM>;
     constexpr int NV = V::NV, NP = V::NP, IE = V::IE, in = NP + d;
     const Cst<float> &C = P.k32;
+    {  // coarse data mostly shows in the pressure already: one variable's work
+       // instead of all where that drops a stencil (leaving a face to the full
+       // evaluation is always right)
+        float D[5], l;
+#pragma unroll
+        for (int k = 0; k < 5; ++k) split_double(S[k + 1][IE] - S[k][IE], D[k], l);
+        if (!teno6a_keeps_all(mk2(D[0], D[4]), mk2(D[1], D[3]), bc2(D[2]))) return false;
+    }
     float Dh[5][NV], Dl[5][NV];
     double val[NV];
     unsigned top = 0;

@@ -1,8 +1,9 @@
 """The double WENO5 sweeps' two face paths -- nonlinear correction and HLLC
 dissipation in float pairs where the stencil is resolved, all double elsewhere
 -- against the oracle, on both sides of the criterion and of the range the
-pairs cover.  Bar: 1e-13 for one right-hand side as it enters one update, the
-bar of the other right-hand-side cases."""
+pairs cover, and the reverse sweep's.  Grids above and below the size from
+which the choice is made face by face.  Bar: 1e-13 for one right-hand side as
+it enters one update, the bar of the other right-hand-side cases."""
 import numpy as np
 import pytest
 
@@ -45,7 +46,7 @@ SCALES = {"unit": dict(rho=(1.0, 0.5), p0=1.0, u0=0.3), "air": dict(rho=(1.2, 0.
 @pytest.mark.parametrize("recon,weno", [("char", "js"), ("char", "z"), ("comp", "js"), ("comp", "z")])
 @pytest.mark.parametrize("scale", list(SCALES))
 def test_single_phase(scale, recon, weno, amp):
-    for ndim, n, bc in ((2, [33, 17], "zerograd"), (3, [9, 7, 11], "symmetry")):
+    for ndim, n, bc in ((2, [33, 17], "zerograd"), (2, [157, 131], "zerograd"), (3, [29, 27, 26], "symmetry")):
         _check(dict(wl.smooth_random(ndim, n, "spm", seed=3, recon=recon, bc=bc, amp=amp, **SCALES[scale]),
                     weno=weno))
 
@@ -54,17 +55,67 @@ def test_single_phase(scale, recon, weno, amp):
 @pytest.mark.parametrize("recon", ["char", "comp"])
 @pytest.mark.parametrize("amp", [1e-4, 0.1])
 def test_five_equation_stiffened(amp, recon, weno):
-    _check(dict(wl.smooth_random(2, [29, 23], "dim", seed=5, recon=recon, amp=amp, limiter=True, gamma=(6.12, 1.4),
+    _check(dict(wl.smooth_random(2, [161, 123], "dim", seed=5, recon=recon, amp=amp, limiter=True, gamma=(6.12, 1.4),
                                  pinf=(3.43e8, 0.0), rho=(1000.0, 1.2), p0=1e5, u0=30.0), weno=weno))
 
 
 def test_resolved_and_unresolved_faces_in_one_warp():
     """A jump in a smooth field: neighbouring faces of a row take both paths,
     at rest (s* = 0) on one side."""
-    case = wl.smooth_random(2, [67, 5], "spm", seed=9, recon="char", bc="zerograd", amp=0.02)
+    case = wl.smooth_random(2, [331, 61], "spm", seed=9, recon="char", bc="zerograd", amp=0.02)
     W = case["W"].copy()
     W[:, :, :, 31:] = W[:, :, :, 31:32]
     W[1:3, :, :, 31:] = 0.0
     W[0, :, :, 31:] *= 0.125
     W[3, :, :, 31:] *= 0.1
     _check(dict(case, W=np.ascontiguousarray(W)))
+
+
+@pytest.mark.parametrize("recon,weno", [("char", "js"), ("char", "z"), ("comp", "js"), ("comp", "z")])
+@pytest.mark.parametrize("amp", [0.02, 0.3])
+@pytest.mark.parametrize("ndim,n,bc", [(2, [163, 121], "symmetry"), (3, [30, 27, 26], "periodic")])
+def test_reverse_sweep_against_the_oracle_tangent(ndim, n, bc, amp, recon, weno):
+    """<Ubar, v> = <Rbar, (dR/dU) v> with the oracle's dual-number tangent, for
+    random Rbar and v, relative to the sum of the products' magnitudes: every
+    term is accurate to about 1e-13 of its own size (the right-hand side's bar)."""
+    case = dict(wl.smooth_random(ndim, n, "spm", seed=21, recon=recon, bc=bc, amp=amp), weno=weno)
+    c = oracle_config(case)
+    U = oracle.prim_to_cons(c, case["W"])
+    rng = np.random.default_rng(22)
+    v, rbar = rng.standard_normal(U.shape), rng.standard_normal(U.shape)
+    _, Rv = oracle.rhs_tangent(c, U, v)
+    s = jxf.Solver(case, "fp64")
+    g = s.rhs_vjp(torch.from_numpy(U).cuda(), torch.from_numpy(rbar).cuda()).cpu().numpy()
+    s.close()
+    a, b = float(np.sum(g * v)), float(np.sum(rbar * Rv))
+    size = float(np.sum(np.abs(g * v)) + np.sum(np.abs(rbar * Rv)))
+    print("<Ubar, v> %.17g, <Rbar, R'v> %.17g, rel %.2e" % (a, b, abs(a - b) / size))
+    assert abs(a - b) < 1e-13 * size
+
+
+def test_level_set_cut_faces_sorted():
+    """The level-set sweep's dry, resolved and unresolved faces (sorted within
+    each block) against the oracle's cut-cell right-hand side."""
+    n, h = [31, 29, 27], 1.0 / 31
+    P = orc_bc = (oracle.PERIODIC, oracle.PERIODIC)
+    ax = np.meshgrid(*[(np.arange(n[e]) + 0.5) * h for e in (2, 1, 0)], indexing="ij")[::-1]
+    phi = 0.3 - np.sqrt(sum((a - 0.5 * a.max()) ** 2 for a in ax))
+    w = 0.02 * np.cos(2 * np.pi * (ax[0] / ax[0].max() + ax[1]))
+    jump = np.where(ax[2] > 0.7 * ax[2].max(), 3.0, 1.0)
+    W = np.stack([(1.0 + w) * jump, 0.3 + w, -0.2 * w, 0.1 + 0 * w, (1.0 + w) * jump])
+    cfg = oracle.make_config(ndim=3, n=n, dx=[h] * 3, bc=[orc_bc] * 3, gamma=(1.4, 1.4), recon=oracle.CHAR)
+    lcfg = oracle.ls_config(ndim=3, n=n, h=h, bc=[P] * 3)
+    ap, al, dg, nr = oracle.ls_geometry(lcfg, phi)
+    ug, pg = np.zeros((3,) + phi.shape), np.where(dg > 0, 1.0, 0.0)
+    grid = jxf.ls_grid(3, n, h, [(jxf.JXF_BC_PERIODIC,) * 2] * 3)
+    eos, sch = jxf.jxf_eos(), jxf.jxf_scheme()
+    eos.gamma[0] = eos.gamma[1] = 1.4
+    sch.recon, sch.weno_eps = jxf.JXF_WENO5JS_CHAR, 1e-6
+    d = [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (ap, dg, nr, W, ug, pg)]
+    dU = torch.zeros(W.shape, dtype=torch.float64, device="cuda")
+    scr = torch.zeros(5 * jxf.jxf_ls_nface(grid), dtype=torch.float64, device="cuda")
+    for phase in (1, 2):
+        ref = oracle.ls_cut_rhs(cfg, phi, W, phase, ug, pg)
+        jxf.jxf_ls_cut_rhs(grid, eos, sch, d[0], d[1], d[2], d[3], phase, d[4], d[5], dU, scr)
+        err = np.abs(dU.cpu().numpy() - ref).max() / np.abs(ref).max()
+        assert err < 1e-13, (phase, err)
