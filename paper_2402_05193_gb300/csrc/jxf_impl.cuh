@@ -816,6 +816,21 @@ __device__ __forceinline__ void teno6a_pair_f2(const float (&x)[6], float &vl, f
                             mul2(mul2(bc2((float)(21520059541.0 / 1377684.0)), a5), a5)))));
     }
     const f2 tau = abs2(sub2(b6, mul2(fma2(bc2(4.f), b[1], add2(b[0], b[2])), bc2((float)(1.0 / 6.0)))));
+    // tau <= 8.9 beta_k for all k makes every gamma_k at least 1 and at most
+    // 9.9^6 in the selection below, so the largest cut-off (1e-7 of their sum)
+    // keeps all four on both sides: their linear combination, without eta and
+    // the selection (8 reciprocals a side).  128^3 viscous vortex
+    // step 1.74 -> 1.22 ms.
+    {
+        const float ml = fminf(fminf(b[0].v.x, b[1].v.x), fminf(b[2].v.x, b[3].v.x)) + 1e-30f;
+        const float mr = fminf(fminf(b[0].v.y, b[1].v.y), fminf(b[2].v.y, b[3].v.y)) + 1e-30f;
+        if (tau.v.x <= 8.9f * ml && tau.v.y <= 8.9f * mr) {
+            const f2 n = fma2(bc2(0.2f), q[3], fma2(bc2(0.05f), q[2], fma2(bc2(0.3f), q[1], mul2(bc2(0.45f), q[0]))));
+            vl = n.v.x;
+            vr = n.v.y;
+            return;
+        }
+    }
     const f2 P[6] = {vm2, vm1, v0, vp1, vp2, vp3};
     const f2 e = bc2((float)kTenoE), two = bc2(2.f);
     float etal = 1.f, etar = 1.f;
@@ -1199,41 +1214,47 @@ __device__ __forceinline__ bool reconstruct_split(const Dev &P, const double (&S
     return true;
 }
 
-// ------------------------------------------- double TENO6-A, all kept ----
-// TENO6-A's selection is sharp: where all four candidates are kept, the value
-// is the linear six-cell interpolation (1, -8, 37, 37, -8, 1)/60, the same from
-// both sides and, being linear, the same in characteristic and in primitive
-// variables.  All are kept when gamma_k >= C_T sum_j gamma_j with the largest
-// cut-off, 1e-7; gamma_k = a_k^6, a_k = 1 + tau6/(beta_k + eps) >= 1, so
-// tau6 <= 9 beta_k for every k is enough (1 >= 4e-7 10^6).  That is told in
-// float from the differences D_k: the indicators are positive definite in
-// them (no difference cancels, relative error below 2e-5, of beta_6 below
-// 6e-5), and a difference too small for float leaves beta below eps, where
-// all are kept as well.  The differences of the characteristic variables can
-// cancel (no entropy or one acoustic wave only): they are projected in float
-// pairs, and where less than 2^-30 of their terms is left the face is not
-// taken.  So a face is taken here only if the double evaluation keeps
-// everything for every variable and side; its double work is then 11
-// operations per variable instead of 260, and with equal states on both sides
-// the HLLC flux is the physical flux.  All other faces are evaluated in double
-// as before.  TENO6-A with 6th-order viscous fluxes, one right-hand side: 64^3
-// periodic vortex 3.23 -> 0.64 ms, 67x58x45 between walls (half of whose faces
-// drop stencils) 2.33 -> 1.06 ms.
+// -------------------------- double TENO6-A, selection told in float ----
+// TENO6-A's selection is sharp: what is kept decides, the face value is then a
+// linear combination of the six cells.  The double evaluation of indicators
+// and selection takes 260 operations per variable; the decision itself is
+// told in float with bounds on its error wherever it is not close:
+//   gamma_k = a_k^6 >= C_T sum_j gamma_j,  a_k = 1 + tau6/(beta_k + eps).
+// The indicators are positive definite in the differences D_k (no difference
+// cancels: relative error below 2e-5, of beta_6 below 6e-5), so tau6 is known
+// to 6e-5 (beta_6 + ...) and every a_k lies in an interval; a candidate is kept
+// (dropped) for certain if it is at the unfavourable ends of all intervals,
+// with the cut-offs of the classes next to eta's.  A difference too small for
+// float leaves beta below eps, where all are kept as well.  The differences of
+// the characteristic variables can cancel (no entropy or one acoustic wave
+// only): they are projected in float pairs, and where less than 2^-30 of their
+// terms is left nothing is told.  So a face is taken here only if the double
+// evaluation selects the same for every variable and side:
+//   all kept everywhere (tau6 <= 9 beta_k is enough: 1 >= 4e-7 10^6): the
+//     six-cell value (1, -8, 37, 37, -8, 1)/60, the same from both sides and,
+//     being linear, in characteristic and in primitive variables -- 11 double
+//     operations per variable, and the HLLC flux of equal states is the
+//     physical flux;
+//   else the kept candidates' combination of the characteristic differences,
+//     in double (about 140 operations in 3-D).
+// Faces with a close decision are evaluated in double as before.  One
+// right-hand side with 6th-order viscous fluxes: 64^3 periodic vortex 3.23 ->
+// 0.39 ms, 67x58x45 between walls 2.33 -> 0.39 ms.
 //
 // Lanes as in teno6a_pair_f2 (the mirrored differences change sign, which the
-// squares do not see).  True if both sides keep all candidates for certain.
-// D0, D1, D2: the pairs (D_0, D_4), (D_1, D_3), (D_2, D_2).
-__device__ __forceinline__ bool teno6a_keeps_all(f2 D0, f2 D1, f2 D2) {
+// squares do not see).  D0, D1, D2: the pairs (D_0, D_4), (D_1, D_3),
+// (D_2, D_2).  b: beta_k, tau: tau6, tol: a bound of its error.
+__device__ __forceinline__ void teno6a_indicators(f2 D0, f2 D1, f2 D2, f2 (&b)[4], f2 &tau, f2 &tol) {
     const f2 D3 = swap2(D1), D4 = swap2(D0);
     const f2 k13 = bc2((float)(13.0 / 12.0)), q = bc2(0.25f);
     auto sq2 = [&](f2 a, f2 c) { return fma2(mul2(k13, a), a, mul2(mul2(q, c), c)); };
-    const f2 b0 = sq2(sub2(D2, D1), add2(D1, D2));
-    const f2 b1 = sq2(sub2(D3, D2), fma2(bc2(-3.f), D2, D3));
-    const f2 b2 = sq2(sub2(D1, D0), fma2(bc2(3.f), D1, neg2(D0)));
+    b[0] = sq2(sub2(D2, D1), add2(D1, D2));
+    b[1] = sq2(sub2(D3, D2), fma2(bc2(-3.f), D2, D3));
+    b[2] = sq2(sub2(D1, D0), fma2(bc2(3.f), D1, neg2(D0)));
     const f2 e1 = fma2(bc2(11.f), D2, fma2(bc2(-7.f), D3, add2(D4, D4)));
     const f2 e2 = fma2(bc2(-2.f), D2, fma2(bc2(3.f), D3, neg2(D4)));
     const f2 e3 = fma2(bc2(-2.f), D3, add2(D2, D4));
-    const f2 b3 = fma2(mul2(bc2((float)(1.0 / 36.0)), e1), e1,
+    b[3] = fma2(mul2(bc2((float)(1.0 / 36.0)), e1), e1,
                        fma2(mul2(k13, e2), e2, mul2(mul2(bc2((float)(781.0 / 720.0)), e3), e3)));
     const f2 a1 = mul2(fma2(bc2(5034.f), D2, fma2(bc2(2444.f), D1, fma2(bc2(-1636.f), D3,
                        fma2(bc2(259.f), D4, mul2(bc2(-341.f), D0))))), bc2((float)(1.0 / 5760.0)));
@@ -1249,52 +1270,131 @@ __device__ __forceinline__ bool teno6a_keeps_all(f2 D0, f2 D1, f2 D2) {
                        fma2(mul2(bc2((float)(781.0 / 20.0)), s3), s3,
                             fma2(mul2(bc2((float)(1421461.0 / 2275.0)), a4), a4,
                                  mul2(mul2(bc2((float)(21520059541.0 / 1377684.0)), a5), a5)))));
-    const f2 bs = mul2(fma2(bc2(4.f), b1, add2(b0, b2)), bc2((float)(1.0 / 6.0)));
-    const f2 tau = abs2(sub2(b6, bs)), tol = mul2(bc2(6e-5f), add2(b6, bs));
+    const f2 bs = mul2(fma2(bc2(4.f), b[1], add2(b[0], b[2])), bc2((float)(1.0 / 6.0)));
+    tau = abs2(sub2(b6, bs));
+    tol = mul2(bc2(6e-5f), add2(b6, bs));
+}
+
+// True if both sides keep all candidates for certain.
+__device__ __forceinline__ bool teno6a_keeps_all(const f2 (&b)[4], f2 tau, f2 tol) {
     const f2 hi = add2(tau, tol);
     // 9 less the indicators' relative error
-    const float ml = 8.5f * (fminf(fminf(b0.v.x, b1.v.x), fminf(b2.v.x, b3.v.x)) + 1e-30f);
-    const float mr = 8.5f * (fminf(fminf(b0.v.y, b1.v.y), fminf(b2.v.y, b3.v.y)) + 1e-30f);
+    const float ml = 8.5f * (fminf(fminf(b[0].v.x, b[1].v.x), fminf(b[2].v.x, b[3].v.x)) + 1e-30f);
+    const float mr = 8.5f * (fminf(fminf(b[0].v.y, b[1].v.y), fminf(b[2].v.y, b[3].v.y)) + 1e-30f);
     return hi.v.x <= ml && hi.v.y <= mr;
 }
 
+// Bit k set: candidate k is kept; -1: not certain.  ct_hi >= ct_lo: the
+// cut-offs eta allows.
+__device__ __forceinline__ int teno6a_mask(float b0, float b1, float b2, float b3, float tau, float tol, float ct_lo,
+                                           float ct_hi) {
+    const float b[4] = {b0, b1, b2, b3};
+    float lo[4], hi[4], mlo = 1.f, mhi = 1.f;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {  // 3e-5: the indicators' error and the reciprocal's
+        lo[k] = 1.f + fmaxf(tau - tol, 0.f) * rcp(fmaf(b[k], 1.00003f, 1.0001e-30f));
+        hi[k] = 1.f + (tau + tol) * rcp(fmaf(b[k], 0.99997f, 0.9999e-30f));
+        mlo = fmaxf(mlo, lo[k]);
+        mhi = fmaxf(mhi, hi[k]);
+    }
+    auto pow6 = [](float x) {
+        const float x2 = x * x;
+        return x2 * x2 * x2;
+    };
+    const float ilo = rcp(mlo), ihi = rcp(mhi);
+    float slo = 0.f, shi = 0.f;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        slo += pow6(lo[k] * ilo);
+        shi += pow6(hi[k] * ihi);
+    }
+    int mask = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {  // 1e-4: rounding of the powers and sums
+        if (pow6(lo[k] * ihi) >= 1.0001f * (ct_hi * shi)) mask |= 1 << k;
+        else if (!(pow6(hi[k] * ilo) * 1.0001f < ct_lo * slo)) return -1;
+    }
+    return mask;
+}
+
+// Masks of both sides of one variable (left | right << 4); -1: not certain.
+__device__ __forceinline__ int teno6a_masks(f2 D0, f2 D1, f2 D2) {
+    f2 b[4], tau, tol;
+    teno6a_indicators(D0, D1, D2, b, tau, tol);
+    if (teno6a_keeps_all(b, tau, tol)) return 0xFF;
+    // eta is the same for both sides: min over neighbouring pairs
+    const float D[5] = {D0.v.x, D1.v.x, D2.v.x, D1.v.y, D0.v.y}, e = (float)kTenoE;
+    float eta = 1.f, big = 0.f;
+#pragma unroll
+    for (int j = 1; j < 5; ++j) {
+        const float p = D[j], m = D[j - 1];
+        eta = fminf(eta, (fabsf(2.f * p * m) + e) * rcp(fmaf(p, p, fmaf(m, m, e))));
+        big = fmaxf(big, fmaxf(fabsf(p), fabsf(m)));
+    }
+    if (!(big < 1e15f)) return -1;
+    auto cls = [](float x) {
+        return (x >= (float)kTenoEta1 ? 1 : 0) + (x >= (float)kTenoEta2 ? 1 : 0) + (x >= (float)kTenoEta3 ? 1 : 0);
+    };
+    const float ct_hi = teno_cutoff<float>(cls(eta * 0.9999f)), ct_lo = teno_cutoff<float>(cls(eta * 1.0001f));
+    const int l = teno6a_mask(b[0].v.x, b[1].v.x, b[2].v.x, b[3].v.x, tau.v.x, tol.v.x, ct_lo, ct_hi);
+    const int r = teno6a_mask(b[0].v.y, b[1].v.y, b[2].v.y, b[3].v.y, tau.v.y, tol.v.y, ct_lo, ct_hi);
+    return l < 0 || r < 0 ? -1 : l | r << 4;
+}
+
+// Face value minus the cell's for the kept candidates of a mask, as
+// coefficients of D_0..D_4: candidates (D1 + 2 D2)/6, (4 D2 - D3)/6,
+// (5 D1 - 2 D0)/6, (9 D2 - 4 D3 + D4)/12 with the weights (9, 6, 1, 4)/20
+// renormalised.
+struct TenoTable {
+    double c[16][5];
+};
+constexpr TenoTable teno_table() {
+    TenoTable t{};
+    const double q[4][5] = {{0, 2, 4, 0, 0}, {0, 0, 8, -2, 0}, {-4, 10, 0, 0, 0}, {0, 0, 9, -4, 1}};  // times 12
+    const double d[4] = {9, 6, 1, 4};
+    for (int m = 1; m < 16; ++m) {
+        double den = 0.0;
+        for (int k = 0; k < 4; ++k)
+            if ((m >> k) & 1) den += d[k];
+        for (int j = 0; j < 5; ++j) {
+            double s = 0.0;
+            for (int k = 0; k < 4; ++k)
+                if ((m >> k) & 1) s += d[k] * q[k][j];
+            t.c[m][j] = s / (12.0 * den);
+        }
+    }
+    return t;
+}
+__device__ const TenoTable kTenoTable = teno_table();
+
+enum { FACE_NONE = -1, FACE_FULL = 0, FACE_SPLIT = 1, FACE_CENTRAL = 2, FACE_TRY = 3 };
+
+// Face states with the selection told in float: FACE_CENTRAL (all kept, equal
+// states), FACE_FULL (combinations of the kept) or FACE_NONE (not certain,
+// nothing written).
 template <int MODEL, int NDIM, int d>
-__device__ __forceinline__ bool reconstruct_central(const Dev &P, const double (&S)[6][MAXV], double *WL, double *WR) {
+__device__ __forceinline__ int reconstruct_teno(const Dev &P, const double (&S)[6][MAXV], double *WL, double *WR) {
     using V = Vars<MODEL, NDIM>;
     constexpr int NV = V::NV, NP = V::NP, IE = V::IE, in = NP + d;
     const Cst<float> &C = P.k32;
-    {  // coarse data mostly shows in the pressure already: one variable's work
-       // instead of all where that drops a stencil (leaving a face to the full
-       // evaluation is always right)
-        float D[5], l;
-#pragma unroll
-        for (int k = 0; k < 5; ++k) split_double(S[k + 1][IE] - S[k][IE], D[k], l);
-        if (!teno6a_keeps_all(mk2(D[0], D[4]), mk2(D[1], D[3]), bc2(D[2]))) return false;
-    }
+    const bool chr = P.recon != JXF_WENO5JS_COMP;
     float Dh[5][NV], Dl[5][NV];
-    double val[NV];
     unsigned top = 0;
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-        double t[5];
 #pragma unroll
         for (int k = 0; k < 6; ++k) top = max(top, (unsigned)__double2hiint(S[k][v]) & 0x7FFFFFFFu);
 #pragma unroll
-        for (int k = 0; k < 5; ++k) {
-            t[k] = S[k + 1][v] - S[k][v];
-            split_double(t[k], Dh[k][v], Dl[k][v]);
-        }
-        // (x2 + x3)/2 plus small terms: one rounding at the value's size
-        const double s1 = t[3] - t[1], s2 = (t[4] - t[0]) + s1;
-        val[v] = S[2][v] + (0.5 * t[2] + (1.0 / 60.0) * (s2 - 8.0 * s1));
+        for (int k = 0; k < 5; ++k) split_double(S[k + 1][v] - S[k][v], Dh[k][v], Dl[k][v]);
     }
-    bool ok = top < 0x47600000u;
+    if (top >= 0x47600000u) return FACE_NONE;
     auto pair = [&](int k, int v) {
         return d2{mk2(Dh[k][v], Dh[4 - k][v]), mk2(Dl[k][v], Dl[4 - k][v])};
     };
-    if (P.recon == JXF_WENO5JS_COMP) {
+    int mask[NV], all = 0xFF;
+    if (!chr) {
 #pragma unroll
-        for (int v = 0; v < NV; ++v) ok = ok && teno6a_keeps_all(pair(0, v).h, pair(1, v).h, pair(2, v).h);
+        for (int v = 0; v < NV; ++v) mask[v] = teno6a_masks(pair(0, v).h, pair(1, v).h, pair(2, v).h);
     } else {
         float wh[NV], wl[NV], rho = 0.f;
 #pragma unroll
@@ -1308,18 +1408,17 @@ __device__ __forceinline__ bool reconstruct_central(const Dev &P, const double (
             const float a1 = wh[V::IA >= 0 ? V::IA : 0];
             rc2 = wh[IE] + (wh[IE] + (C.B2h + a1 * C.dBh)) * rcp(C.A2h + a1 * C.dAh);
         }
-        ok = ok && rho > 1.5e-5f && rho < 1e10f && rc2 > 1.5e-5f && rc2 < 1e18f;
-        if (!ok) return false;
+        if (!(rho > 1.5e-5f && rho < 1e10f && rc2 > 1.5e-5f && rc2 < 1e18f)) return FACE_NONE;
         const Frozen<MODEL, NDIM> fz(C, wh, wl, Dh[2], Dl[2]);
-        // q = x + y (the pairs): all kept, and not cancelled beyond the pairs' accuracy
-        auto keeps = [&](const d2 (&q)[3], const f2 (&size)[3]) {
+        // q: the selection, unless cancelled beyond the pairs' accuracy
+        auto masks = [&](const d2 (&q)[3], const f2 (&size)[3]) {
             float m = 0.f, r = 0.f;
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
                 m = fmaxf(m, fmaxf(fabsf(q[k].h.v.x), fabsf(q[k].h.v.y)));
                 r = fmaxf(r, fmaxf(size[k].v.x, size[k].v.y));
             }
-            return m >= 9.3e-10f * r && teno6a_keeps_all(q[0].h, q[1].h, q[2].h);
+            return m >= 9.3e-10f * r ? teno6a_masks(q[0].h, q[1].h, q[2].h) : -1;
         };
         d2 qi[3], qe[3];
         f2 sz[3];
@@ -1330,7 +1429,8 @@ __device__ __forceinline__ bool reconstruct_central(const Dev &P, const double (
             qi[k] = renorm(dsub(b, a));
             sz[k] = add2(abs2(a.h), abs2(b.h));
         }
-        ok = keeps(qe, sz) && keeps(qi, sz);
+        mask[IE] = masks(qe, sz);
+        mask[in] = masks(qi, sz);
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
             if (v == in || v == IE) continue;
@@ -1343,16 +1443,96 @@ __device__ __forceinline__ bool reconstruct_central(const Dev &P, const double (
                     q[k] = renorm(dsub(a, b));
                     sz[k] = add2(abs2(a.h), abs2(b.h));
                 }
-                ok = ok && keeps(q, sz);
+                mask[v] = masks(q, sz);
             } else {
-                ok = ok && teno6a_keeps_all(pair(0, v).h, pair(1, v).h, pair(2, v).h);
+                mask[v] = teno6a_masks(pair(0, v).h, pair(1, v).h, pair(2, v).h);
             }
         }
     }
-    if (!ok) return false;
 #pragma unroll
-    for (int v = 0; v < NV; ++v) WL[v] = WR[v] = val[v];
-    return true;
+    for (int v = 0; v < NV; ++v) {
+        if (mask[v] < 0) return FACE_NONE;
+        all &= mask[v];
+    }
+    if (all == 0xFF) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            // (x2 + x3)/2 plus small terms: one rounding at the value's size
+            const double t1 = S[2][v] - S[1][v], t2 = S[3][v] - S[2][v], t3 = S[4][v] - S[3][v];
+            const double s1 = t3 - t1, s2 = ((S[5][v] - S[4][v]) - (S[1][v] - S[0][v])) + s1;
+            WL[v] = WR[v] = S[2][v] + (0.5 * t2 + (1.0 / 60.0) * (s2 - 8.0 * s1));
+        }
+        return FACE_CENTRAL;
+    }
+    // the kept candidates' value minus the cell's, left from D_0.., right from
+    // the mirrored -D_4..
+    auto offsets = [&](const double (&q)[5], int m, double &l, double &r) {
+        const double *cl = kTenoTable.c[m & 15], *cr = kTenoTable.c[m >> 4];
+        l = cl[0] * q[0];
+        r = cr[0] * q[4];
+#pragma unroll
+        for (int j = 1; j < 5; ++j) {
+            l = fma(cl[j], q[j], l);
+            r = fma(cr[j], q[4 - j], r);
+        }
+        r = -r;
+    };
+    auto diff = [&](int v, double (&D)[5]) {
+#pragma unroll
+        for (int k = 0; k < 5; ++k) D[k] = S[k + 1][v] - S[k][v];
+    };
+    if (!chr) {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            double D[5], l, r;
+            diff(v, D);
+            offsets(D, mask[v], l, r);
+            WL[v] = S[2][v] + l;
+            WR[v] = S[3][v] + r;
+        }
+        return FACE_FULL;
+    }
+    double Wb[MAXV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) Wb[v] = 0.5 * (S[2][v] + S[3][v]);
+    const double rho = density_of<double, MODEL, NDIM>(Wb);
+    Eos<double, MODEL> eos(P, alpha_of<double, MODEL, NDIM>(Wb));
+    const double rc2 = eos.rc2_from_p(P, Wb[IE]);
+    const double t = rsq(rho * rc2), c = rc2 * t, rt = rho * t, irc2 = rt * t, hc = 0.5 * rt, hr = 0.5 * irc2;
+    double Du[5], Dp[5], li, ri, le, re;
+    diff(in, Du);
+    diff(IE, Dp);
+    {
+        double qi[5], qe[5];
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+            const double a = hc * Du[k], b = hr * Dp[k];
+            qe[k] = b + a;
+            qi[k] = b - a;
+        }
+        offsets(qe, mask[IE], le, re);
+        offsets(qi, mask[in], li, ri);
+    }
+    const double sl = li + le, sr = ri + re;
+    WL[in] = S[2][in] + c * (le - li);
+    WR[in] = S[3][in] + c * (re - ri);
+    WL[IE] = S[2][IE] + rc2 * sl;
+    WR[IE] = S[3][IE] + rc2 * sr;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+        if (v == in || v == IE) continue;
+        double q[5], l, r;
+        diff(v, q);
+        if (v < NP) {
+            const double ent = Wb[v] * irc2;
+#pragma unroll
+            for (int k = 0; k < 5; ++k) q[k] = fma(-ent, Dp[k], q[k]);
+        }
+        offsets(q, mask[v], l, r);
+        WL[v] = S[2][v] + (v < NP ? fma(Wb[v], sl, l) : l);
+        WR[v] = S[3][v] + (v < NP ? fma(Wb[v], sr, r) : r);
+    }
+    return FACE_FULL;
 }
 
 // ------------------------------------------------------ reconstruction ----
@@ -1430,10 +1610,9 @@ __device__ __forceinline__ void reconstruct_w(const Dev &P, const T (&S)[6][MAXV
 // weights, chosen per face from P.weno_z), 2: TENO6-A (its own kernels, so
 // that its registers do not weigh on the WENO5 sweeps).
 // HOW a double face is reconstructed: all in double, with the split
-// correction (the caller knows it is resolved), or TRY: TENO6-A by the central
-// value if all candidates are kept for certain, WENO5 split if resolved.
+// correction (the caller knows it is resolved), or TRY: TENO6-A with the
+// selection made in float if that is certain, WENO5 split if resolved.
 // Returns how it was, FACE_NONE if a TENO6-A face tried is not certain.
-enum { FACE_NONE = -1, FACE_FULL = 0, FACE_SPLIT = 1, FACE_CENTRAL = 2, FACE_TRY = 3 };
 template <typename T, int MODEL, int NDIM, int d, int RSV, int HOW>
 __device__ __forceinline__ int reconstruct(const Dev &P, const T (&S)[6][MAXV], T *WL, T *WR) {
     if constexpr (std::is_same<T, double>::value && HOW == FACE_SPLIT) {
@@ -1441,7 +1620,7 @@ __device__ __forceinline__ int reconstruct(const Dev &P, const T (&S)[6][MAXV], 
         return FACE_SPLIT;
     }
     if constexpr (std::is_same<T, double>::value && HOW == FACE_TRY && RSV == 2)
-        return reconstruct_central<MODEL, NDIM, d>(P, S, WL, WR) ? FACE_CENTRAL : FACE_NONE;
+        return reconstruct_teno<MODEL, NDIM, d>(P, S, WL, WR);
     if constexpr (std::is_same<T, double>::value && HOW == FACE_TRY && RSV != 2 && NDIM > 1)
         if (P.split && reconstruct_split<MODEL, NDIM, d, true>(P, S, WL, WR)) return FACE_SPLIT;
     if constexpr (RSV == 2) reconstruct_w<T, MODEL, NDIM, d, 2>(P, S, WL, WR);
