@@ -30,7 +30,9 @@ template <typename T, int MODEL, int NDIM, int VH, int RSV> void launch_flux(con
 
 template <typename T, int MODEL, int NDIM, int VH, int RSV>
 void launch_flux_update(const Dev &P, int epi, cudaStream_t s) {
-    if constexpr (NDIM >= 2 && std::is_same<T, float>::value) {
+    if constexpr (NDIM == 1) {
+        k_line_update<T, MODEL, VH, RSV><<<fused_grid(P, 1), kFluxThreads, 0, s>>>(P, epi);
+    } else if constexpr (std::is_same<T, float>::value) {
         const dim3 grid = fused_grid(P, NDIM);
         k_flux_update<T, MODEL, NDIM, VH, RSV><<<grid, kFluxThreads, 0, s>>>(P, epi, fused_run(P, NDIM));
     }

@@ -33,7 +33,7 @@ struct jxf_ctx {
     void *F[3] = {nullptr, nullptr, nullptr}, *UH[3] = {nullptr, nullptr, nullptr};
     void *G = nullptr;  // per-cell auxiliary arrays: velocity gradient (viscous) or THINC normal
     int naux = 0;       // their count
-    // fused last-axis sweep (ndim >= 2, whole grids): the stage writes its
+    // fused last-axis sweep (float, and 1-D grids): the stage writes its
     // primitives and temperature to the next of three buffers and its state
     // to a buffer the stage does not read
     int fused = 0;
@@ -646,7 +646,7 @@ jxf_status create_handle(const jxf_grid *grid, const jxf_eos *eos, const jxf_sch
     if (blk) {
         // cell arrays with three halo planes on each side of the split axis
         const size_t vs = (size_t)P.vstride * h->esize, off = 3 * plane * h->esize;
-        h->fused = h->ndim >= 2 && h->esize == 4 ? 1 : 0;
+        h->fused = h->ndim == 1 || h->esize == 4 ? 1 : 0;
         const size_t nvr = (size_t)h->nv, f = (size_t)h->fused;
         void **dst[10] = {&h->Un, &h->Us, &h->W, &h->Tt, &h->G, &h->W2, &h->W3, &h->T2, &h->T3, &h->Us2};
         const size_t rows[10] = {nvr, nvr, nvr, 1, (size_t)h->naux, f * nvr, f * nvr, f, f, f * nvr};
@@ -669,7 +669,7 @@ jxf_status create_handle(const jxf_grid *grid, const jxf_eos *eos, const jxf_sch
         chk(dalloc(h, &h->W, sb));
         chk(dalloc(h, &h->Tt, (size_t)ncell * h->esize));
         if (h->naux) chk(dalloc(h, &h->G, (size_t)h->naux * ncell * h->esize));
-        if (h->ndim >= 2 && h->esize == 4) {  // the fused last-axis sweep's rotating buffers (float)
+        if (h->ndim == 1 || h->esize == 4) {  // the fused last-axis sweep's rotating buffers
             h->fused = 1;
             chk(dalloc(h, &h->W2, sb));
             chk(dalloc(h, &h->W3, sb));

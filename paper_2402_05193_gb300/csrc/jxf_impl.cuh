@@ -2952,11 +2952,10 @@ __device__ __forceinline__ float warp_min_keyed(float v) { return warp_min(v); }
 // variable instead of 47 in double; in float the only double operation per
 // variable is the last one).  k_prim on 256x128x128 five-equation cells in
 // float 275 -> 45 us, on 128^3 in double 308 -> 184 us.
-template <typename T, int NV>
+template <typename T, int NV, int NT = kCellThreads>
 __device__ __forceinline__ void block_partials(const Dev &P, T smax, T rmin, bool bad, const T *U, double *out) {
-    constexpr int NW = kCellThreads / 32;
-    static_assert(NV < NW, "one warp per variable and one for the rest");
-    __shared__ T buf[NV][kCellThreads];
+    constexpr int NW = NT / 32;
+    __shared__ T buf[NV][NT];
     __shared__ T sh_max[NW], sh_min[NW];
     __shared__ int sh_bad[NW];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -2971,8 +2970,8 @@ __device__ __forceinline__ void block_partials(const Dev &P, T smax, T rmin, boo
         sh_bad[wid] = anybad ? 1 : 0;
     }
     __syncthreads();
-    if (wid < NV) {
-        const T *b = buf[wid] + lane;
+    for (int v = wid; v < NV; v += NW) {
+        const T *b = buf[v] + lane;
         double s;
         if constexpr (sizeof(T) == 8) {
             T a = b[0];
@@ -2990,8 +2989,9 @@ __device__ __forceinline__ void block_partials(const Dev &P, T smax, T rmin, boo
             }
             s = warp_sum_pairs_to_double(hi, lo);
         }
-        if (lane == 0) out[3 + wid] = s * P.vol;
-    } else if (wid == NW - 1 && lane == 0) {
+        if (lane == 0) out[3 + v] = s * P.vol;
+    }
+    if (wid == NW - 1 && lane == 0) {
         T a = sh_max[0], b = sh_min[0];
         int c = sh_bad[0];
 #pragma unroll
@@ -3046,6 +3046,32 @@ __device__ __forceinline__ void finish_cell(const Dev &P, long long i, const T *
     bad = !ok;
 }
 
+// RK stage combination Uout = ca Un + cb Us + cc dt R of cell ic, its new
+// primitives and the epilogue quantities.
+template <typename T, int MODEL, int NDIM>
+__device__ __forceinline__ void combine_cell(const Dev &P, T cdt, int ic, const T *R, int epi, T *U, T &smax, T &rmin,
+                                             bool &bad) {
+    constexpr int NV = Vars<MODEL, NDIM>::NV;
+    const size_t nc = (size_t)P.vstride;
+    const T *Un = static_cast<const T *>(P.Un);
+    const T *Us = static_cast<const T *>(P.Us);
+    T *Uo = static_cast<T *>(P.Uout);
+    const bool first = P.stage0 != 0;  // stage 1: U1 = Un + dt R
+    const T ca = first ? T(0) : (sizeof(T) == 8 ? T(P.ca) : T(P.ca32)), cb = sizeof(T) == 8 ? T(P.cb) : T(P.cb32);
+    T un[MAXV], us[MAXV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {  // all loads before any store (Uout may alias)
+        us[v] = (Us + v * nc)[ic];
+        un[v] = first ? T(0) : (Un + v * nc)[ic];
+    }
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+        U[v] = first ? us[v] + cdt * R[v] : ca * un[v] + cb * us[v] + cdt * R[v];
+        (Uo + v * nc)[ic] = U[v];
+    }
+    finish_cell<T, MODEL, NDIM>(P, ic, U, epi, smax, rmin, bad);
+}
+
 // --------------------------------------------------------------- k_update --
 // The work of one cell i: divergence of the face fluxes (+ the a1 div(u)
 // source), then mode 0: dU = R; mode 1: stage combination Uout = ca Un +
@@ -3096,23 +3122,7 @@ __device__ __forceinline__ void update_cell(const Dev &P, T cdt, long long i, in
         for (int v = 0; v < NV; ++v) (dU + v * nc)[ic] = R[v];
         return;
     }
-    const T *Un = static_cast<const T *>(P.Un);
-    const T *Us = static_cast<const T *>(P.Us);
-    T *Uo = static_cast<T *>(P.Uout);
-    const bool first = P.stage0 != 0;  // stage 1: U1 = Un + dt R
-    const T ca = first ? T(0) : (sizeof(T) == 8 ? T(P.ca) : T(P.ca32)), cb = sizeof(T) == 8 ? T(P.cb) : T(P.cb32);
-    T un[MAXV], us[MAXV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {  // all loads before any store (Uout may alias)
-        us[v] = (Us + v * nc)[ic];
-        un[v] = first ? T(0) : (Un + v * nc)[ic];
-    }
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-        U[v] = first ? us[v] + cdt * R[v] : ca * un[v] + cb * us[v] + cdt * R[v];
-        (Uo + v * nc)[ic] = U[v];
-    }
-    finish_cell<T, MODEL, NDIM>(P, i, U, epi, smax, rmin, bad);
+    combine_cell<T, MODEL, NDIM>(P, cdt, ic, R, epi, U, smax, rmin, bad);
 }
 
 // c dt of the stage in the storage type, computed once per block.
@@ -3297,6 +3307,60 @@ __global__ void __launch_bounds__(kFluxThreads, FusedMinBlocks<T, RSV>::value)
     }
 }
 
+// ------------------------------------------------- 1-D stage in one kernel --
+// The faces and the cell update of one RK stage of a 1-D grid: a block
+// computes kLineCells + 1 faces (one of them again in the next block, counted
+// there), hands the fluxes over in shared memory and updates its cells, in the
+// arithmetic of the separate kernels.  1-D runs are bound by latency, a chain
+// of double instructions at 64 clocks each and the kernels' own start and end:
+// 200-cell tube 65 -> @LINE@ us a step.  Reads W / Tt / Ucell, writes Wout / Tout /
+// Uout, which must not alias them.
+constexpr int kLineCells = kFluxThreads - 1;
+template <typename T, int MODEL, int VH, int RSV>
+__global__ void __launch_bounds__(kFluxThreads, SweepMinBlocks<T, RSV>::value) k_line_update(const Dev P, const int epi) {
+    using V = Vars<MODEL, 1>;
+    constexpr int NV = V::NV;
+    __shared__ T sF[NV][kFluxThreads], sH[kFluxThreads];
+    double dt;
+    if (!block_dt(P, dt)) return;
+    const T cdt = block_cdt<T>(P, dt);
+    const int tid = threadIdx.x, n = P.n[0], i = (int)blockIdx.x * kLineCells + tid;  // face i, cell i
+    bool il = false, fl = false;
+    if (i <= n) {
+        const int c[3] = {i, 0, 0};
+        const bool count = tid < kLineCells || i == n;
+        T F[MAXV], uh;
+        bool done = false;
+        if constexpr (std::is_same<T, double>::value && RSV == 2)
+            done = flux_face_at<T, MODEL, 1, 0, VH, RSV, FACE_TRY>(P, dt, c, count, F, uh, il, fl);
+        if (!done) flux_face_at<T, MODEL, 1, 0, VH, RSV, FACE_FULL>(P, dt, c, count, F, uh, il, fl);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) sF[v][tid] = F[v];
+        if (MODEL == JXF_DIM) sH[tid] = uh;
+    }
+    if (P.limiter) count_limited(P, il, fl);
+    __syncthreads();
+    T smax = T(0), rmin = T(3e38), U[MAXV];
+    bool bad = false;
+#pragma unroll
+    for (int v = 0; v < NV; ++v) U[v] = T(0);
+    if (tid < kLineCells && i < n) {
+        const T idx = cst<T>(P).inv_dx[0];
+        T R[NV];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            R[v] = T(0);
+            R[v] -= (sF[v][tid + 1] - sF[v][tid]) * idx;
+        }
+        if constexpr (MODEL == JXF_DIM) {
+            const T a1 = (static_cast<const T *>(P.Us) + V::IA * (size_t)P.vstride)[i];
+            R[V::IA] += a1 * (sH[tid + 1] - sH[tid]) * idx;
+        }
+        combine_cell<T, MODEL, 1>(P, cdt, i, R, epi, U, smax, rmin, bad);
+    }
+    if (epi) block_partials<T, NV, kFluxThreads>(P, smax, rmin, bad, U, P.part + (size_t)blockIdx.x * (3 + MAXV));
+}
+
 // Primitives (+ temperature) of a conservative state, with the reduction
 // epilogue (used after the state is set).
 template <typename T, int MODEL, int NDIM>
@@ -3369,22 +3433,77 @@ constexpr int kPartThreads = 32;
 // clipped at t_end.  mode 0: partials -> diagnostics + dt; mode 1: the same
 // after a step (advance t by the step's dt first); mode 2: re-clip dt from
 // the stored diagnostics (after the time was set).
-constexpr int kFinalThreads = 32;
+//
+// Latency-bound (a dependent double instruction takes 64 clocks): four warps,
+// one per FP64 pipe, share the records, extrema go over the integer pipe and
+// each sum's four parts are added by a lane of its own.  512 records 6.1 ->
+// @FIN@ us (one warp before).
+constexpr int kFinalThreads = 128;
 __device__ __forceinline__ void finalize_block(const Dev &P, const double *part, int npart, int nv,
                                                int mode) {
-    const int t = threadIdx.x;
+    constexpr int NW = kFinalThreads / 32;
+    __shared__ double s_sum[NW][MAXV];
+    __shared__ long long s_max[NW], s_min[NW];
+    __shared__ int s_bad[NW];
+    const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
     double *sc = P.scal;
     const double dt_cur = sc[SC_DT];
     if (mode == 1 && !(dt_cur > 0.0)) return;  // finished: the step did nothing
-    double a[3 + MAXV];
-    if (mode != 2 && t < 32) reduce_records(part, 0, npart, nv, a);
-    if (t != 0) return;
     if (mode != 2) {
-        sc[SC_SMAX] = a[0];
-        sc[SC_RMIN] = a[1];
-        for (int v = 0; v < nv; ++v) sc[SC_SUMS + v] = a[3 + v];
-        if (a[2] > 0.0) *P.status |= ST_NONPHYSICAL;
+        long long kmax = order_key(__double_as_longlong(-1e300)), kmin = order_key(__double_as_longlong(1e300));
+        int bad = 0;
+        double a[MAXV];
+#pragma unroll
+        for (int v = 0; v < MAXV; ++v) a[v] = 0.0;
+        auto number = [](long long b) { return (b & 0x7FFFFFFFFFFFFFFFLL) <= 0x7FF0000000000000LL; };
+#pragma unroll 2
+        for (int b = t; b < npart; b += kFinalThreads) {
+            const double *p = part + (size_t)b * (3 + MAXV);
+            const long long x = __double_as_longlong(p[0]), y = __double_as_longlong(p[1]);
+            if (number(x)) kmax = max(kmax, order_key(x));
+            if (number(y)) kmin = min(kmin, order_key(y));
+            bad |= __double_as_longlong(p[2]) > 0 ? 1 : 0;
+#pragma unroll
+            for (int v = 0; v < MAXV; ++v)
+                if (v < nv) a[v] += p[3 + v];
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            kmax = max(kmax, __shfl_down_sync(0xffffffffu, kmax, o));
+            kmin = min(kmin, __shfl_down_sync(0xffffffffu, kmin, o));
+#pragma unroll
+            for (int v = 0; v < MAXV; ++v)
+                if (v < nv) a[v] += __shfl_down_sync(0xffffffffu, a[v], o);
+        }
+        bad = __any_sync(0xffffffffu, bad);
+        if (lane == 0) {
+            s_max[wid] = kmax;
+            s_min[wid] = kmin;
+            s_bad[wid] = bad;
+#pragma unroll
+            for (int v = 0; v < MAXV; ++v) s_sum[wid][v] = a[v];
+        }
+        __syncthreads();
+        if (t < nv) {
+            double s = s_sum[0][t];
+#pragma unroll
+            for (int w = 1; w < NW; ++w) s += s_sum[w][t];
+            sc[SC_SUMS + t] = s;
+        }
+        if (t == 0) {
+            int b = 0;
+#pragma unroll
+            for (int w = 0; w < NW; ++w) {
+                kmax = max(kmax, s_max[w]);
+                kmin = min(kmin, s_min[w]);
+                b |= s_bad[w];
+            }
+            sc[SC_SMAX] = __longlong_as_double(order_key(kmax));
+            sc[SC_RMIN] = __longlong_as_double(order_key(kmin));
+            if (b) *P.status |= ST_NONPHYSICAL;
+        }
     }
+    if (t != 0) return;
     if (mode == 1) {
         sc[SC_T] += dt_cur;
         sc[SC_DT_LAST] = dt_cur;

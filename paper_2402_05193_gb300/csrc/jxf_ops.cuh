@@ -8,7 +8,7 @@ namespace jxf {
 
 struct Ops {
     void (*flux)(const Dev &, int d, cudaStream_t);
-    // the last axis's faces fused with the stage update (ndim >= 2)
+    // the last axis's faces fused with the stage update (float, and 1-D grids)
     void (*flux_update)(const Dev &, int epi, cudaStream_t);
     void (*update)(const Dev &, int mode, int epi, cudaStream_t);
     void (*prim)(const Dev &, int epi, cudaStream_t);
@@ -51,6 +51,7 @@ inline int fused_run(const Dev &P, int ndim) {
     return run;
 }
 inline dim3 fused_grid(const Dev &P, int ndim) {
+    if (ndim == 1) return dim3(grid_for(P.n[0], kLineCells));  // k_line_update
     const long long plane = (long long)P.n[0] * (ndim == 3 ? P.n[1] : 1);
     const int run = fused_run(P, ndim);
     return dim3(grid_for(plane, kFluxThreads), (unsigned)((P.n[ndim - 1] + run - 1) / run));
