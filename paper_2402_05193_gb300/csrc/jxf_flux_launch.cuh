@@ -31,7 +31,14 @@ template <typename T, int MODEL, int NDIM, int VH, int RSV> void launch_flux(con
 template <typename T, int MODEL, int NDIM, int VH, int RSV>
 void launch_flux_update(const Dev &P, int epi, cudaStream_t s) {
     if constexpr (NDIM == 1) {
-        k_line_update<T, MODEL, VH, RSV><<<fused_grid(P, 1), kFluxThreads, 0, s>>>(P, epi);
+        constexpr int G = kLaneGroup<Vars<MODEL, 1>::NV>;
+        if constexpr (std::is_same<T, double>::value && RSV != 2) {
+            if (P.line_group == G) {
+                k_line_update<T, MODEL, VH, RSV, G><<<fused_grid(P, 1), kFluxThreads, 0, s>>>(P, epi);
+                return;
+            }
+        }
+        k_line_update<T, MODEL, VH, RSV, 1><<<fused_grid(P, 1), kFluxThreads, 0, s>>>(P, epi);
     } else if constexpr (std::is_same<T, float>::value) {
         const dim3 grid = fused_grid(P, NDIM);
         k_flux_update<T, MODEL, NDIM, VH, RSV><<<grid, kFluxThreads, 0, s>>>(P, epi, fused_run(P, NDIM));

@@ -145,6 +145,7 @@ struct Dev {
     int weno_z;  // 0: Jiang-Shu weights, 1: WENO5-Z weights
     int teno;    // 1: TENO6-A instead of WENO5
     int viscous, limiter;
+    int line_group;  // 1-D grids: lanes per face (see k_line_update)
     int split;   // double WENO5: resolved faces take the split correction (see kSplitFaces)
     int visc_half;  // viscous stencils: points per side (1, 2, 3 for order 2, 4, 6)
     int thinc;   // THINC volume-fraction reconstruction (five-equation model)
@@ -1367,7 +1368,7 @@ constexpr TenoTable teno_table() {
 }
 __device__ const TenoTable kTenoTable = teno_table();
 
-enum { FACE_NONE = -1, FACE_FULL = 0, FACE_SPLIT = 1, FACE_CENTRAL = 2, FACE_TRY = 3 };
+enum { FACE_NONE = -1, FACE_FULL = 0, FACE_SPLIT = 1, FACE_CENTRAL = 2, FACE_TRY = 3, FACE_LANES = 4 };
 
 // Face states with the selection told in float: FACE_CENTRAL (all kept, equal
 // states), FACE_FULL (combinations of the kept) or FACE_NONE (not certain,
@@ -1583,9 +1584,9 @@ __device__ __forceinline__ void reconstruct_w(const Dev &P, const T (&S)[6][MAXV
         for (int j = 0; j < 6; ++j) {
             const T *w = S[j];
             T val;
-            if (v < NP) val = w[v] - ent[v] * w[IE];
-            else if (v == IE) val = h_c * w[in] + h_rc2 * w[IE];
-            else if (v == in) val = -h_c * w[in] + h_rc2 * w[IE];
+            if (v < NP) val = fma(-ent[v], w[IE], w[v]);
+            else if (v == IE) val = fma(h_c, w[in], h_rc2 * w[IE]);
+            else if (v == in) val = fma(-h_c, w[in], h_rc2 * w[IE]);
             else val = w[v];
             q[j] = val;
         }
@@ -1609,12 +1610,80 @@ __device__ __forceinline__ void reconstruct_w(const Dev &P, const T (&S)[6][MAXV
 // RSV: the kernel variant's scheme family -- 0: WENO5 (Jiang-Shu or Z
 // weights, chosen per face from P.weno_z), 2: TENO6-A (its own kernels, so
 // that its registers do not weigh on the WENO5 sweeps).
+// reconstruct_w() of a double WENO5 face by a group of G neighbouring lanes
+// that hold the same stencil: lane k of the group does the weights of variable
+// k, then all share the values (the same operations, so the same bits).  Where
+// one warp's chain of double instructions is what takes the time (1-D grids),
+// this shortens it by the variables' number.  All lanes of the warp call.
+template <int NV> constexpr int kLaneGroup = NV <= 4 ? 4 : 8;
+template <int MODEL, int NDIM, int d, bool Z>
+__device__ __forceinline__ void reconstruct_lanes(const Dev &P, const double (&S)[6][MAXV], double *WL, double *WR) {
+    using V = Vars<MODEL, NDIM>;
+    constexpr int NV = V::NV, NP = V::NP, IE = V::IE, in = NP + d, G = kLaneGroup<NV>;
+    const int k = (int)(threadIdx.x & (G - 1)), v = k < NV ? k : 0, first = (int)(threadIdx.x & 31) - k;
+    const bool chr = P.recon != JXF_WENO5JS_COMP;
+    auto mine = [&](const double *w) {  // w[v] by selection (registers)
+        double x = w[0];
+#pragma unroll
+        for (int u = 1; u < NV; ++u) x = v == u ? w[u] : x;
+        return x;
+    };
+    double Wb[MAXV], ent[2] = {0.0, 0.0}, cb = 0.0, rc2 = 0.0, h_c = 0.0, h_rc2 = 0.0, q[6];
+    if (chr) {
+#pragma unroll
+        for (int u = 0; u < NV; ++u) Wb[u] = 0.5 * (S[2][u] + S[3][u]);
+        const double rho = density_of<double, MODEL, NDIM>(Wb);
+        Eos<double, MODEL> eos(P, alpha_of<double, MODEL, NDIM>(Wb));
+        rc2 = eos.rc2_from_p(P, Wb[IE]);
+        const double t = rsq(rho * rc2), rt = rho * t, irc2 = rt * t;
+        cb = rc2 * t;
+        h_c = 0.5 * rt;
+        h_rc2 = 0.5 * irc2;
+#pragma unroll
+        for (int u = 0; u < NP; ++u) ent[u] = Wb[u] * irc2;
+        const bool ac = v == in || v == IE, part = v < NP;
+        const double a = part ? -(v == 0 ? ent[0] : ent[NP - 1]) : (v == in ? -h_c : h_c);
+#pragma unroll
+        for (int j = 0; j < 6; ++j) {
+            const double x = ac ? h_rc2 * S[j][IE] : mine(S[j]), y = part ? S[j][IE] : S[j][in];
+            q[j] = ac || part ? fma(a, y, x) : x;
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < 6; ++j) q[j] = mine(S[j]);
+    }
+    double ql, qr;
+    weno5_pair<Z>(q, P.k64.weno_eps4, ql, qr);
+#pragma unroll
+    for (int u = 0; u < NV; ++u) {
+        WL[u] = __shfl_sync(0xffffffffu, ql, first + u);
+        WR[u] = __shfl_sync(0xffffffffu, qr, first + u);
+    }
+    if (!chr) return;
+    double *outs[2] = {WL, WR};
+#pragma unroll
+    for (int s = 0; s < 2; ++s) {
+        double *o = outs[s];
+        const double qi = o[in], qe = o[IE];
+#pragma unroll
+        for (int u = 0; u < NP; ++u) o[u] = Wb[u] * qi + o[u] + Wb[u] * qe;
+        o[in] = cb * (qe - qi);
+        o[IE] = rc2 * (qi + qe);
+    }
+}
+
 // HOW a double face is reconstructed: all in double, with the split
 // correction (the caller knows it is resolved), or TRY: TENO6-A with the
 // selection made in float if that is certain, WENO5 split if resolved.
-// Returns how it was, FACE_NONE if a TENO6-A face tried is not certain.
+// LANES: all in double, by a group of lanes.  Returns how it was, FACE_NONE
+// if a TENO6-A face tried is not certain.
 template <typename T, int MODEL, int NDIM, int d, int RSV, int HOW>
 __device__ __forceinline__ int reconstruct(const Dev &P, const T (&S)[6][MAXV], T *WL, T *WR) {
+    if constexpr (std::is_same<T, double>::value && HOW == FACE_LANES) {
+        if (P.weno_z) reconstruct_lanes<MODEL, NDIM, d, true>(P, S, WL, WR);
+        else reconstruct_lanes<MODEL, NDIM, d, false>(P, S, WL, WR);
+        return FACE_FULL;
+    }
     if constexpr (std::is_same<T, double>::value && HOW == FACE_SPLIT) {
         reconstruct_split<MODEL, NDIM, d, false>(P, S, WL, WR);
         return FACE_SPLIT;
@@ -3308,35 +3377,47 @@ __global__ void __launch_bounds__(kFluxThreads, FusedMinBlocks<T, RSV>::value)
 }
 
 // ------------------------------------------------- 1-D stage in one kernel --
-// The faces and the cell update of one RK stage of a 1-D grid: a block
-// computes kLineCells + 1 faces (one of them again in the next block, counted
-// there), hands the fluxes over in shared memory and updates its cells, in the
-// arithmetic of the separate kernels.  1-D runs are bound by latency, a chain
-// of double instructions at 64 clocks each and the kernels' own start and end:
-// 200-cell tube 65 -> @LINE@ us a step.  Reads W / Tt / Ucell, writes Wout / Tout /
-// Uout, which must not alias them.
-constexpr int kLineCells = kFluxThreads - 1;
-template <typename T, int MODEL, int VH, int RSV>
+// The faces and the cell update of one RK stage of a 1-D grid: a block of
+// kFluxThreads / G groups of G lanes computes one face per group (its last
+// face again in the next block, counted there), hands the fluxes over in
+// shared memory and updates the cells between, in the arithmetic of the
+// separate kernels.  1-D runs are bound by latency, a chain of double
+// instructions at 64 clocks each and the kernels' own start and end: G > 1
+// lanes share a double face's WENO weights (reconstruct_lanes) while every warp
+// has an FP64 pipe to itself (up to 4712 cells single-phase, 2280
+// five-equation; beyond, the lanes' common work would cost more than it
+// saves: 4800 cells 68 us a step in groups, 62 without).  200-cell tube, us a
+// step: 65 as two kernels, 58 fused, 40 with groups.  Reads W / Tt / Ucell,
+// writes Wout / Tout / Uout, which must not alias them.
+template <typename T, int MODEL, int VH, int RSV, int G>
 __global__ void __launch_bounds__(kFluxThreads, SweepMinBlocks<T, RSV>::value) k_line_update(const Dev P, const int epi) {
     using V = Vars<MODEL, 1>;
-    constexpr int NV = V::NV;
-    __shared__ T sF[NV][kFluxThreads], sH[kFluxThreads];
+    constexpr int NV = V::NV, kFaces = kFluxThreads / G;
+    __shared__ T sF[NV][kFaces], sH[kFaces];
     double dt;
     if (!block_dt(P, dt)) return;
     const T cdt = block_cdt<T>(P, dt);
-    const int tid = threadIdx.x, n = P.n[0], i = (int)blockIdx.x * kLineCells + tid;  // face i, cell i
+    const int tid = threadIdx.x, n = P.n[0], base = (int)blockIdx.x * (kFaces - 1);
     bool il = false, fl = false;
-    if (i <= n) {
-        const int c[3] = {i, 0, 0};
-        const bool count = tid < kLineCells || i == n;
-        T F[MAXV], uh;
-        bool done = false;
-        if constexpr (std::is_same<T, double>::value && RSV == 2)
-            done = flux_face_at<T, MODEL, 1, 0, VH, RSV, FACE_TRY>(P, dt, c, count, F, uh, il, fl);
-        if (!done) flux_face_at<T, MODEL, 1, 0, VH, RSV, FACE_FULL>(P, dt, c, count, F, uh, il, fl);
+    {
+        const int k = tid / G, f = base + k;  // face f, lane tid % G of its group
+        const bool lead = tid % G == 0 && f <= n;
+        const int c[3] = {min(f, n), 0, 0};  // idle groups go along: the group exchange takes whole warps
+        const bool count = lead && (k < kFaces - 1 || f == n);
+        T F[MAXV], uh = T(0);
+        if constexpr (G > 1) {
+            flux_face_at<T, MODEL, 1, 0, VH, RSV, FACE_LANES>(P, dt, c, count, F, uh, il, fl);
+        } else if (lead) {
+            bool done = false;
+            if constexpr (std::is_same<T, double>::value && RSV == 2)
+                done = flux_face_at<T, MODEL, 1, 0, VH, RSV, FACE_TRY>(P, dt, c, count, F, uh, il, fl);
+            if (!done) flux_face_at<T, MODEL, 1, 0, VH, RSV, FACE_FULL>(P, dt, c, count, F, uh, il, fl);
+        }
+        if (lead) {
 #pragma unroll
-        for (int v = 0; v < NV; ++v) sF[v][tid] = F[v];
-        if (MODEL == JXF_DIM) sH[tid] = uh;
+            for (int v = 0; v < NV; ++v) sF[v][k] = F[v];
+            if (MODEL == JXF_DIM) sH[k] = uh;
+        }
     }
     if (P.limiter) count_limited(P, il, fl);
     __syncthreads();
@@ -3344,7 +3425,8 @@ __global__ void __launch_bounds__(kFluxThreads, SweepMinBlocks<T, RSV>::value) k
     bool bad = false;
 #pragma unroll
     for (int v = 0; v < NV; ++v) U[v] = T(0);
-    if (tid < kLineCells && i < n) {
+    const int i = base + tid;  // cell
+    if (tid < kFaces - 1 && i < n) {
         const T idx = cst<T>(P).inv_dx[0];
         T R[NV];
 #pragma unroll
@@ -3436,8 +3518,8 @@ constexpr int kPartThreads = 32;
 //
 // Latency-bound (a dependent double instruction takes 64 clocks): four warps,
 // one per FP64 pipe, share the records, extrema go over the integer pipe and
-// each sum's four parts are added by a lane of its own.  512 records 6.1 ->
-// @FIN@ us (one warp before).
+// each sum's four parts are added by a lane of its own.  With its launch 6.1 ->
+// 5.4 us (one warp before).
 constexpr int kFinalThreads = 128;
 __device__ __forceinline__ void finalize_block(const Dev &P, const double *part, int npart, int nv,
                                                int mode) {

@@ -51,7 +51,7 @@ inline int fused_run(const Dev &P, int ndim) {
     return run;
 }
 inline dim3 fused_grid(const Dev &P, int ndim) {
-    if (ndim == 1) return dim3(grid_for(P.n[0], kLineCells));  // k_line_update
+    if (ndim == 1) return dim3(grid_for(P.n[0], kFluxThreads / P.line_group - 1));  // k_line_update
     const long long plane = (long long)P.n[0] * (ndim == 3 ? P.n[1] : 1);
     const int run = fused_run(P, ndim);
     return dim3(grid_for(plane, kFluxThreads), (unsigned)((P.n[ndim - 1] + run - 1) / run));

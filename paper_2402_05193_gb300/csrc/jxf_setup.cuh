@@ -119,6 +119,13 @@ inline void fill_dev(const jxf_grid *grid, const jxf_eos *eos, const jxf_scheme 
     P.thinc = scheme->thinc && eos->model == JXF_DIM ? 1 : 0;
     P.limiter = scheme->limiter ? 1 : 0;
     const bool f64 = scheme->precision == JXF_FP64;
+    // 1-D double WENO5: a group of lanes per face as long as every block then has
+    // an SM, and every warp an FP64 pipe, to itself
+    const int group = eos->model == JXF_DIM ? kLaneGroup<5> : kLaneGroup<3>;
+    P.line_group = grid->ndim == 1 && f64 && !P.teno &&
+                           grid->n[0] <= 152 * (kFluxThreads / group - 1)
+                       ? group
+                       : 1;
     // by the whole grid, also for a block of it: the blocks' faces are evaluated
     // as the grid's
     for (int d = 0; d < grid->ndim; ++d) {
