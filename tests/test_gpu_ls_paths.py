@@ -82,3 +82,43 @@ def test_extension_from_a_band(steps):
     scr = torch.full((4 * phi.size,), 7.0, dtype=torch.float64, device="cuda")
     jxf.jxf_ls_extend(grid, *d, 4, 2, steps, scr)
     assert np.abs(d[4].cpu().numpy() - ref).max() < 1e-13
+
+
+@pytest.mark.parametrize("ndim,n,centre", [(2, [50, 40], (1, 2)), (2, [256, 9], (255, 4)), (3, [24, 21, 18], (0, 20, 1)),
+                                           (3, [17, 64, 5], (8, 33, 2)), (3, [6, 6, 90], (3, 3, 0))])
+def test_extension_leaves_out_empty_blocks(ndim, n, centre):
+    """A small drop, most blocks of the grid empty and its band reaching others
+    along each axis and across the periodic sides: the interface quantities
+    that jxf_ls_init extends are those of jxf_ls_interface and the plain
+    extension (20 convex combinations: 1e-13 of the largest value)."""
+    h, bc, gamma, pinf = 1.0 / 16, [(P, P)] * ndim, (1.4, 1.67), (0.0, 0.3)
+    grid = jxf.ls_grid(ndim, n, h, bc)
+    dist = []
+    for e in range(ndim):
+        x = np.abs(np.arange(n[e]) - centre[e] + 0.25)
+        dist.append(np.minimum(x, n[e] - x) * h)
+    mesh = np.meshgrid(*dist[::-1], indexing="ij")
+    phi = 1.6 * h - np.sqrt(sum(m * m for m in mesh))
+    rng = np.random.default_rng(5)
+    W = [torch.from_numpy(rng.uniform(0.5, 1.5, (ndim + 2,) + phi.shape)).cuda() for _ in range(2)]
+    eos = []
+    for k in range(2):
+        e = jxf.jxf_eos()
+        e.model = jxf.JXF_SPM
+        e.gamma[0] = e.gamma[1] = gamma[k]
+        e.pinf[0] = e.pinf[1] = pinf[k]
+        eos.append(e)
+    sch = jxf.jxf_scheme()
+    sch.recon, sch.precision, sch.weno_eps = jxf.JXF_WENO5JS_CHAR, jxf.JXF_FP64, 1e-6
+    d = torch.from_numpy(np.ascontiguousarray(phi)).cuda()
+    z = lambda k: torch.zeros((k,) + phi.shape, dtype=torch.float64, device="cuda")
+    got = z(ndim + 1)
+    work = torch.full((jxf.jxf_ls_step_work(grid),), 3.0, dtype=torch.float64, device="cuda")
+    jxf.jxf_ls_init(grid, *eos, sch, d, *W, z(ndim + 2), z(ndim + 2), got, work)
+    ap = torch.zeros(jxf.jxf_ls_nface(grid), dtype=torch.float64, device="cuda")
+    al, dg, nr, want = z(1)[0], z(1)[0], z(ndim), z(ndim + 1)
+    jxf.jxf_ls_geometry(grid, d, ap, al, dg, nr)
+    jxf.jxf_ls_interface(grid, *W, gamma, pinf, al, dg, nr, want[:ndim], want[ndim])
+    jxf.jxf_ls_extend(grid, d, al, dg, nr, want, ndim + 1, 2, 20, z(ndim + 1))
+    assert want.abs().max() > 0.1
+    assert (got - want).abs().max() < 1e-13 * want.abs().max()
