@@ -334,7 +334,8 @@ jxf_status jxf_batch_set_time(jxf_batch b, int sim, double t, jxf_stream stream)
 jxf_status jxf_batch_get_state(jxf_batch b, int sim, void *U, jxf_stream stream);
 /* Tile shape of the face sweeps: tile_faces (a multiple of 128) faces per
  * tile, persistent grid of blocks_per_sm blocks per SM (0: one block per
- * tile).  Picked by the autotuner (paper_2402_05193_gb300.autotune). */
+ * tile).  Picked by the autotuner (paper_2402_05193_gb300.autotune); without
+ * this call by the number of faces (512, 256 or 128 per tile, 128 in double). */
 jxf_status jxf_batch_set_tiling(jxf_batch b, int tile_faces, int blocks_per_sm);
 /* n RK3 steps of every simulation (queued on the stream, one graph launch). */
 jxf_status jxf_batch_step(jxf_batch b, int n, jxf_stream stream);
@@ -350,9 +351,10 @@ const char *jxf_batch_last_error(jxf_batch b);
  * accumulate per kind k: ms[k] += device time, launches[k] += kernels
  * launched, for k = 0, 1, 2: face sweeps along x, y, z; 3: cell update (and
  * the auxiliary pass after it, where the scheme has one); 4: step
- * finalisation (its one or two kernels).  5 entries each, caller-owned host
- * arrays.  Synchronises the stream after every step; returns the status of
- * the device check. */
+ * finalisation (its one or two kernels).  A kernel that does the last axis's
+ * sweep and the update counts under 2 (float storage, 2-D and 3-D) or 0 (1-D).
+ * 5 entries each, caller-owned host arrays.  Synchronises the stream once, at
+ * the end; returns the status of the device check. */
 jxf_status jxf_step_profiled(jxf_handle h, int n, float *ms, int *launches, jxf_stream stream);
 
 /* Host-side fault injection (tests of the failure paths): the k-th device

@@ -296,7 +296,7 @@ void fused_stage(jxf_ctx *h, Dev &P, int stage, cudaStream_t s, KernelTimer *kt)
         h->ops->flux(P, d, s);
         if (kt) kt->end(s);
     }
-    if (kt) kt->begin(2, s);
+    if (kt) kt->begin(h->ndim == 1 ? 0 : 2, s);  // 1-D: the x sweep
     h->ops->flux_update(P, stage == 2 ? 1 : 0, s);
     if (kt) kt->end(s);
 }
