@@ -1298,6 +1298,9 @@ __device__ __forceinline__ int teno6a_mask(float b0, float b1, float b2, float b
         mlo = fmaxf(mlo, lo[k]);
         mhi = fmaxf(mhi, hi[k]);
     }
+    // beside a flat sub-stencil a_k reaches tau6/1e-30 (a 2 kPa step in Pa gives
+    // 2^126): above, the reciprocal below would be flushed to 0 and keep everything
+    if (!(mhi < 8e37f)) return -1;
     auto pow6 = [](float x) {
         const float x2 = x * x;
         return x2 * x2 * x2;

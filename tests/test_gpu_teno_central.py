@@ -65,3 +65,22 @@ def test_cancelling_characteristics(kind):
 def test_five_equation(recon):
     _check(dict(wl.smooth_random(2, [41, 37], "dim", seed=13, recon=recon, amp=0.02, limiter=True, gamma=(1.4, 1.66),
                                  rho=(1.2, 0.17), p0=1e5, u0=30.0), weno="teno6a"))
+
+
+@pytest.mark.parametrize("n,axis", [((1170,), 0), ((1170, 5), 0), ((5, 1170), 1)])
+@pytest.mark.parametrize("recon", ["comp", "char"])
+def test_jumps_between_constant_states(recon, n, axis):
+    """Steps of 1e3 to 2e4 in data in physical units (pressure component-wise,
+    density where the characteristic variables carry it), up and down, at every
+    place of a block of 128 faces: beside flat cells tau6/beta spans float's
+    range, and only the flat side may be kept."""
+    ndim = len(n)
+    J = np.geomspace(1e3, 2e4, 65)
+    q = np.full(130, 1e5)
+    q[1::2] += J
+    q = np.repeat(q, 9).reshape([n[axis] if e == axis else 1 for e in (2, 1, 0)])
+    case = wl.smooth_random(ndim, list(n), "spm", seed=1, recon=recon, bc="zerograd", amp=0.0)
+    W = np.empty_like(case["W"])
+    W[0], W[1:1 + ndim], W[1 + ndim] = 1.2, 3.0, 1e5
+    W[0 if recon == "char" else 1 + ndim] = q
+    _check(dict(case, W=W, weno="teno6a"))
