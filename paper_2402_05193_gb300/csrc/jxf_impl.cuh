@@ -1223,14 +1223,16 @@ __device__ __forceinline__ bool reconstruct_split(const Dev &P, const double (&S
 //   gamma_k = a_k^6 >= C_T sum_j gamma_j,  a_k = 1 + tau6/(beta_k + eps).
 // The indicators are positive definite in the differences D_k (no difference
 // cancels: relative error below 2e-5, of beta_6 below 6e-5), so tau6 is known
-// to 6e-5 (beta_6 + ...) and every a_k lies in an interval; a candidate is kept
+// to 7.5e-5 (beta_6 + ...) and every a_k lies in an interval; a candidate is kept
 // (dropped) for certain if it is at the unfavourable ends of all intervals,
 // with the cut-offs of the classes next to eta's.  A difference too small for
 // float leaves beta below eps, where all are kept as well.  The differences of
 // the characteristic variables can cancel (no entropy or one acoustic wave
-// only): they are projected in float pairs, and where less than 2^-30 of their
-// terms is left nothing is told.  So a face is taken here only if the double
-// evaluation selects the same for every variable and side:
+// only): they are projected in float pairs, and where a pair of neighbouring
+// ones is less than 2^-20 of its terms nothing is told.  So a face is taken here
+// only if the selection of the exact differences is certain for every variable
+// and side (the double evaluation, whose projected values carry 2^-53 of their
+// size, can itself select otherwise where the differences are not much more):
 //   all kept everywhere (tau6 <= 9 beta_k is enough: 1 >= 4e-7 10^6): the
 //     six-cell value (1, -8, 37, 37, -8, 1)/60, the same from both sides and,
 //     being linear, in characteristic and in primitive variables -- 11 double
@@ -1273,7 +1275,7 @@ __device__ __forceinline__ void teno6a_indicators(f2 D0, f2 D1, f2 D2, f2 (&b)[4
                                  mul2(mul2(bc2((float)(21520059541.0 / 1377684.0)), a5), a5)))));
     const f2 bs = mul2(fma2(bc2(4.f), b[1], add2(b[0], b[2])), bc2((float)(1.0 / 6.0)));
     tau = abs2(sub2(b6, bs));
-    tol = mul2(bc2(6e-5f), add2(b6, bs));
+    tol = mul2(bc2(7.5e-5f), add2(b6, bs));
 }
 
 // True if both sides keep all candidates for certain.
@@ -1414,15 +1416,17 @@ __device__ __forceinline__ int reconstruct_teno(const Dev &P, const double (&S)[
         }
         if (!(rho > 1.5e-5f && rho < 1e10f && rc2 > 1.5e-5f && rc2 < 1e18f)) return FACE_NONE;
         const Frozen<MODEL, NDIM> fz(C, wh, wl, Dh[2], Dl[2]);
-        // q: the selection, unless cancelled beyond the pairs' accuracy
+        // q: the selection.  The pairs are good to 2^-44 of the terms (size).  Told
+        // only where that is at most 2^-24 of the larger of any two neighbouring
+        // differences (every sub-stencil holds such a pair): at most 66 times as
+        // much in a beta_k (4e-6) and 196 times in beta_6 (1.2e-5)
         auto masks = [&](const d2 (&q)[3], const f2 (&size)[3]) {
-            float m = 0.f, r = 0.f;
+            const float a[5] = {fabsf(q[0].h.v.x), fabsf(q[1].h.v.x), fabsf(q[2].h.v.x), fabsf(q[1].h.v.y), fabsf(q[0].h.v.y)};
+            const float r[5] = {size[0].v.x, size[1].v.x, size[2].v.x, size[1].v.y, size[0].v.y};
+            bool known = true;
 #pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                m = fmaxf(m, fmaxf(fabsf(q[k].h.v.x), fabsf(q[k].h.v.y)));
-                r = fmaxf(r, fmaxf(size[k].v.x, size[k].v.y));
-            }
-            return m >= 9.3e-10f * r ? teno6a_masks(q[0].h, q[1].h, q[2].h) : -1;
+            for (int k = 0; k < 4; ++k) known = known && fmaxf(a[k], a[k + 1]) >= 9.6e-7f * fmaxf(r[k], r[k + 1]);
+            return known ? teno6a_masks(q[0].h, q[1].h, q[2].h) : -1;
         };
         d2 qi[3], qe[3];
         f2 sz[3];
