@@ -119,3 +119,46 @@ def test_level_set_cut_faces_sorted():
         jxf.jxf_ls_cut_rhs(grid, eos, sch, d[0], d[1], d[2], d[3], phase, d[4], d[5], dU, scr)
         err = np.abs(dU.cpu().numpy() - ref).max() / np.abs(ref).max()
         assert err < 1e-13, (phase, err)
+
+
+def _bump(weno, recon, weno_eps):
+    """Parabolic bumps with a small step at their rim in an otherwise exactly
+    uniform state: differences are 0 or well above rounding."""
+    case = wl.smooth_random(2, [157, 131], "spm", seed=4, recon=recon, bc="periodic", amp=0.0)
+    W = case["W"].copy()
+    for v, (cx, cy, a) in enumerate(((40, 30, 0.02), (90, 70, 0.01), (60, 95, -0.01), (110, 40, 0.02))):
+        y, x = np.meshgrid(np.arange(131) - cy, np.arange(157) - cx, indexing="ij")
+        r2 = (x * x + y * y) / 400.0
+        W[v, 0] += np.where(r2 < 1.0, a * (1.05 - r2), 0.0)
+    return dict(case, W=W, weno=weno, weno_eps=weno_eps)
+
+
+@pytest.mark.parametrize("weno_eps", [1e-12, 1e-22, 1e-40, 1e-60])
+@pytest.mark.parametrize("recon,weno", [("char", "js"), ("char", "z"), ("comp", "js"), ("comp", "z")])
+def test_small_weno_eps(recon, weno, weno_eps):
+    """A weight parameter near or below float's range, forward and reverse, in
+    uniform regions (indicators 0) as well."""
+    case = _bump(weno, recon, weno_eps)
+    c = oracle_config(case, weno_eps=weno_eps)
+    U = oracle.prim_to_cons(c, case["W"])
+    dt = oracle.dt(c, U)
+    R_ref, _ = oracle.rhs(c, U, 0.5 * dt)
+    rng = np.random.default_rng(23)
+    v, rbar = rng.standard_normal(U.shape), rng.standard_normal(U.shape)
+    _, Rv = oracle.rhs_tangent(c, U, v)
+    s = jxf.Solver(case, "fp64")
+    R = s.rhs(torch.from_numpy(U).cuda(), 0.5 * dt).cpu().numpy()
+    g = s.rhs_vjp(torch.from_numpy(U).cuda(), torch.from_numpy(rbar).cuda()).cpu().numpy()
+    s.close()
+    err = rhs_update_err(R, R_ref, U, dt, momentum_slice(case))
+    assert np.isfinite(R).all()
+    assert err.max() < TOL, err
+    # beside uniform cells the weights' derivatives cancel over 1/weno_eps: below
+    # 1e-12 the oracle's own tangent loses more than the bar and WENO5-Z's
+    # all-double reverse is large itself; the size of Jiang-Shu's is left
+    assert np.isfinite(g).all()
+    if weno == "js":
+        assert np.abs(g).max() < 1e8
+    a, b = float(np.sum(g * v)), float(np.sum(rbar * Rv))
+    if weno_eps >= 1e-12:
+        assert abs(a - b) < 1e-13 * float(np.sum(np.abs(g * v)) + np.sum(np.abs(rbar * Rv)))
