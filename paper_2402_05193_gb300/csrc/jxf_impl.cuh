@@ -883,13 +883,20 @@ __device__ __forceinline__ void recon_face(const T (&x)[6], T eps4, T &vl, T &vr
 //   left value  = x2 + (D1 + 2 D2 - (2 w_0 T_0 + w_2 T_1))/6,
 //   right value = x3 - (D3 + 2 D2 - (2 w_0 T_2 + w_2 T_1))/6:
 // the weights only multiply T.  Where the stencil is resolved -- |D_k| <=
-// 2^-4 and |T_k| <= 2^-7 of the variable's scale (rho, c, rho c^2, 1) -- this
+// 2^-4 and |T_k| <= 2^-7 of the variable's scale -- this
 // correction is carried in pairs of floats (an unevaluated sum hi + lo; its
-// error against exact arithmetic is 2^-50 of max |T| in the mean and 2^-45 at
-// most, so below 2^-52 of the scale and typically 2^-57), and so is its sum
-// with D1 + 2 D2 (2^-50 of |D| in the mean): together below the rounding of
-// the double face value.  The differences themselves and the sum with the
-// cell value are double.
+// error against exact arithmetic is 2^-50 of max |D| in the mean).  The scale is
+// the value itself for densities, partial densities and volume fraction and
+// rho c^2 for the pressure; there the sum with D1 + 2 D2 is in pairs as well (at
+// most 3/16 of the scale).  Velocities cross zero in smooth flow: D up to c/16, T
+// up to c/128, D1 + 2 D2 in double.  The normal one meets the pressure's own
+// rounding, 2^-53 c, in every flux; a transverse one meets nothing but itself,
+// so its T is also held against its own largest value (kSplitOwn).  Where that
+// fails the face (five-equation model: that velocity) is all double.  The
+// differences and the sum with the cell value, one rounding, are double.
+// Right-hand sides against quadruple precision, mean error of each variable over
+// the all-double formula's, 161 x 141 and 30 x 28 x 27, Mach 0.001 to 1, smooth, 20
+// cells a wave and rough, trace gas, stiffened liquid: 0.13 to 1.03.
 // Other faces (shocks, interfaces, coarse waves) take the double formula
 // above; there the correction form would lose digits next to a jump (the
 // middle candidate's share of the jump cancels).  The choice is made per face
@@ -902,10 +909,8 @@ __device__ __forceinline__ void recon_face(const T (&x)[6], T eps4, T &vl, T &vr
 // shock-bubble 231 | 257, 24^3 waves 244 | 320, 200-cell tube 70 | 73.  With the
 // second warp per pipe the double formula takes twice as long: 160^2 bubble
 // 405 | 298, 160^2 waves 254 | 85, 40^3 815 | 295.
-// FP64 instructions of a 3-D viscous face: 620 -> 117; 128^3 Taylor-Green
-// step 24.8 -> 7.4 ms (sweeps 2.49 -> 0.60 ms each); right-hand sides against
-// float64 references are as close as before (1.1e-14 -> 0.9e-14 on smooth
-// 3-D fields).  Three blocks of 128 an SM (168 registers) let the integer and
+// FP64 instructions of a 3-D viscous face: 620 -> 130; 128^3 Taylor-Green
+// step 24.8 -> 7.6 ms.  Three blocks of 128 an SM (168 registers) let the integer and
 // FP32 work of one warp run beside the FP64 work of the others: 8.75 ms
 // against 9.18 with two and 9.09 with four.
 //
@@ -1028,9 +1033,15 @@ __device__ __forceinline__ double widen(float x) {
     return __hiloint2double((int)((((b & 0x7FFFFFFFu) >> 3) + 0x38000000u) | (b & 0x80000000u)), (int)(b << 29));
 }
 
+// A high word's magnitude (sign removed, below 2^120) truncated to float.
+__device__ __forceinline__ float high_float(unsigned a) {
+    return a < 0x38100000u ? 0.f : __uint_as_float(((a << 3) ^ 0x40000000u) & 0x7FFFFFFFu);
+}
+
 constexpr long long kSplitFaces = 4 * 152 * 32 + 1;
 constexpr float kSplitD = 1.f / 16.f;   // bound of |D| over the variable's scale
 constexpr float kSplitT = 1.f / 128.f;  // bound of |T|
+constexpr float kSplitOwn = 1.f / 16.f;  // bound of a transverse velocity's |T| over its largest value
 
 // The frozen state of a face in float pairs: mean of its two cells, S2 + D2/2
 // (wh, wl: S2; Dh, Dl: D2), with what the projection and its inverse need.
@@ -1069,14 +1080,26 @@ template <int MODEL, int NDIM> struct Frozen {
     }
 };
 
-// Whether a face takes the split correction: largest |D| and |T| of each
-// variable (dm, tm), the state w2 of cell 2 and the stencil's largest high
-// word `top` against the bounds; scales in the range in which the float pairs
-// are normal numbers.
-template <int MODEL, int NDIM>
+// A transverse velocity (nothing couples it to the pressure, so its own size
+// counts, not c) is resolved by itself: |T| against its largest value; below
+// 2^-44 c it is rounding noise of the pressure (2^-53 c an update).
+template <int MODEL, int NDIM, int d> __host__ __device__ constexpr bool split_across(int v) {
+    constexpr int NP = Vars<MODEL, NDIM>::NP;
+    return v >= NP && v < NP + NDIM && v != NP + d;
+}
+__device__ __forceinline__ bool split_own(float tm, float big, float c) {
+    return tm <= fmaxf(kSplitOwn * big, 5.7e-14f * c);
+}
+
+// Whether a face along axis d takes the split correction: largest |D| and |T|
+// of each variable (dm, tm), the state w2 of cell 2, the largest |x| of each
+// variable (big) and the stencil's largest high word `top` against the bounds;
+// scales in the range in which the float pairs are normal numbers.
+template <int MODEL, int NDIM, int d>
 __device__ __forceinline__ bool split_bounds(const Dev &P, const float (&dm)[Vars<MODEL, NDIM>::NV],
                                              const float (&tm)[Vars<MODEL, NDIM>::NV],
-                                             const float (&w2)[Vars<MODEL, NDIM>::NV], unsigned top) {
+                                             const float (&w2)[Vars<MODEL, NDIM>::NV],
+                                             const float (&big)[Vars<MODEL, NDIM>::NV], unsigned top) {
     using V = Vars<MODEL, NDIM>;
     constexpr int NV = V::NV, NP = V::NP, IE = V::IE;
     const Cst<float> &C = P.k32;
@@ -1094,8 +1117,9 @@ __device__ __forceinline__ bool split_bounds(const Dev &P, const float (&dm)[Var
     const float qlim = 7e12f * C.weno_eps4;
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
-        const float sc = v < NP ? rho : (v == IE ? rc2 : (v == V::IA ? 1.f : c));
+        const float sc = v < NP || v == V::IA ? fabsf(w2[v]) : (v == IE ? rc2 : c);
         ok = ok && dm[v] <= kSplitD * sc && tm[v] <= kSplitT * sc;
+        if (split_across<MODEL, NDIM, d>(v) && MODEL == JXF_SPM) ok = ok && split_own(tm[v], big[v], c);
         if (!chr) ok = ok && dm[v] * dm[v] <= qlim;
         else ok = ok && (v == IE ? 0.01f : (kSplitD * kSplitD * 4.f) * sc * sc) <= qlim;
     }
@@ -1112,7 +1136,7 @@ __device__ __forceinline__ void split_sizes(float D0, float D1, float D2, float 
 template <int MODEL, int NDIM, int d, class Hi>
 __device__ __forceinline__ bool face_resolved(const Dev &P, Hi hi) {
     constexpr int NV = Vars<MODEL, NDIM>::NV;
-    float dm[NV], tm[NV], w2[NV];
+    float dm[NV], tm[NV], w2[NV], big[NV];
     unsigned top = 0;
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
@@ -1126,9 +1150,27 @@ __device__ __forceinline__ bool face_resolved(const Dev &P, Hi hi) {
             x[j] = a < 0x38100000u ? 0.f : __uint_as_float(b);
         }
         w2[v] = x[2];
+        big[v] = fmaxf(fmaxf(fmaxf(fabsf(x[0]), fabsf(x[1])), fmaxf(fabsf(x[2]), fabsf(x[3]))), fmaxf(fabsf(x[4]), fabsf(x[5])));
         split_sizes(x[1] - x[0], x[2] - x[1], x[3] - x[2], x[4] - x[3], x[5] - x[4], dm[v], tm[v]);
     }
-    return split_bounds<MODEL, NDIM>(P, dm, tm, w2, top);
+    return split_bounds<MODEL, NDIM, d>(P, dm, tm, w2, big, top);
+}
+
+// The double values of one variable.  A call: inlined it weighs on the
+// registers of every face.
+static __device__ __noinline__ double2 weno5_pair_of(bool z, double eps4, double a, double b, double c, double d, double e,
+                                                     double f) {
+    const double x[6] = {a, b, c, d, e, f};
+    double2 o;
+    if (z) weno5_pair<true>(x, eps4, o.x, o.y);
+    else weno5_pair<false>(x, eps4, o.x, o.y);
+    return o;
+}
+__device__ __forceinline__ void weno5_pair_call(bool z, double eps4, double a, double b, double c, double d, double e,
+                                                double f, double &l, double &r) {
+    const double2 o = weno5_pair_of(z, eps4, a, b, c, d, e, f);
+    l = o.x;
+    r = o.y;
 }
 
 // Face states of a double WENO5 face by the split correction; TRY: if the
@@ -1151,16 +1193,23 @@ __device__ __forceinline__ bool reconstruct_split(const Dev &P, const double (&S
 #pragma unroll
     for (int v = 0; v < NV; ++v)
         if (v < NP || v == IE || v == V::IA) split_double(S[2][v], wh[v], wl[v]);
+    auto largest = [&](int v) {  // largest high word of |x|
+        unsigned a = 0;
+#pragma unroll
+        for (int j = 0; j < 6; ++j) a = max(a, (unsigned)__double2hiint(S[j][v]) & 0x7FFFFFFFu);
+        return a;
+    };
     if constexpr (TRY) {
-        float dm[NV], tm[NV];
+        float dm[NV], tm[NV], big[NV];
         unsigned top = 0;
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
-#pragma unroll
-            for (int j = 0; j < 6; ++j) top = max(top, (unsigned)__double2hiint(S[j][v]) & 0x7FFFFFFFu);
+            const unsigned a = largest(v);
+            top = max(top, a);
+            big[v] = high_float(a);
             split_sizes(Dh[0][v], Dh[1][v], Dh[2][v], Dh[3][v], Dh[4][v], dm[v], tm[v]);
         }
-        if (!split_bounds<MODEL, NDIM>(P, dm, tm, wh, top)) return false;
+        if (!split_bounds<MODEL, NDIM, d>(P, dm, tm, wh, big, top)) return false;
     }
 
     auto pair = [&](int k, int v) {
@@ -1168,12 +1217,29 @@ __device__ __forceinline__ bool reconstruct_split(const Dev &P, const double (&S
     };
     auto swp = [](d2 a) { return d2{swap2(a.h), swap2(a.l)}; };
     auto put = [&](int v, d2 o) {
-        // D1 + 2 D2 less the correction is small next to the cell value: kept
-        // in pairs until the sum with it
+        if (v >= NP && v < NP + NDIM) {  // velocities cross 0, where D1 + 2 D2 is as large as they are: in double
+            if constexpr (MODEL == JXF_DIM) {
+                if (split_across<MODEL, NDIM, d>(v)) {
+                    float dm, tm;
+                    split_sizes(Dh[0][v], Dh[1][v], Dh[2][v], Dh[3][v], Dh[4][v], dm, tm);
+                    if (!split_own(tm, high_float(largest(v)), 0.f)) {
+                        weno5_pair_call(z, P.k64.weno_eps4, S[0][v], S[1][v], S[2][v], S[3][v], S[4][v], S[5][v], WL[v], WR[v]);
+                        return;
+                    }
+                }
+            }
+            const double D = S[3][v] - S[2][v];
+            const double l = fma(2.0, D, S[2][v] - S[1][v]), r = fma(2.0, D, S[4][v] - S[3][v]);
+            WL[v] = fma(1.0 / 6.0, l - (widen(o.h.v.x) + widen(o.l.v.x)), S[2][v]);
+            WR[v] = fma(-1.0 / 6.0, r - (widen(o.h.v.y) + widen(o.l.v.y)), S[3][v]);
+            return;
+        }
+        // D1 + 2 D2 less the correction is at most 3/16 of the cell value (of
+        // rho c^2 for the pressure): kept in pairs until the sum with it
         const d2 D2 = pair(2, v);
         const d2 e = renorm(dsub(dadd(pair(1, v), dscale(D2, bc2(2.f))), o));
-        WL[v] = fma(1.0 / 6.0, widen(e.h.v.x), fma(1.0 / 6.0, widen(e.l.v.x), S[2][v]));
-        WR[v] = fma(-1.0 / 6.0, widen(e.h.v.y), fma(-1.0 / 6.0, widen(e.l.v.y), S[3][v]));
+        WL[v] = fma(1.0 / 6.0, widen(e.h.v.x) + widen(e.l.v.x), S[2][v]);
+        WR[v] = fma(-1.0 / 6.0, widen(e.h.v.y) + widen(e.l.v.y), S[3][v]);
     };
     if (!chr) {
 #pragma unroll

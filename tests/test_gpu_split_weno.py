@@ -162,3 +162,50 @@ def test_small_weno_eps(recon, weno, weno_eps):
     a, b = float(np.sum(g * v)), float(np.sum(rbar * Rv))
     if weno_eps >= 1e-12:
         assert abs(a - b) < 1e-13 * float(np.sum(np.abs(g * v)) + np.sum(np.abs(rbar * Rv)))
+
+
+def test_trace_partial_density_and_volume_fraction():
+    """A rough trace gas carried at the speed of sound: partial density and
+    volume fraction, 1e-4 of the mixture's, are accurate to their own size.  Bar
+    of one update: 8 roundings of 2^-53 in each of two faces' fluxes and in the
+    oracle's, times dt u/dx <= 0.2."""
+    case = wl.smooth_random(2, [161, 141], "dim", seed=5, recon="comp", amp=0.02, gamma=(1.4, 1.66), rho=(1.0, 1.0))
+    W = case["W"].copy()
+    a = 1e-4 * (1.0 + 0.5 * np.random.default_rng(7).uniform(-1, 1, W.shape[1:]))
+    W[0], W[1], W[5], W[2], W[3] = a, 1.0 - a, a, 1.0 + W[2] - 0.3, 0.3
+    for recon in ("comp", "char"):
+        c = oracle_config(dict(case, W=W, recon=recon))
+        U = oracle.prim_to_cons(c, W)
+        dt = oracle.dt(c, U)
+        ref, _ = oracle.rhs(c, U, 0.5 * dt)
+        s = jxf.Solver(dict(case, W=W, recon=recon), "fp64")
+        R = s.rhs(torch.from_numpy(U).cuda(), 0.5 * dt).cpu().numpy()
+        s.close()
+        err = rhs_update_err(R, ref, U, dt)
+        print(recon, err)
+        assert err[[0, 5]].max() < 8 * 2 * 2 * 2.0 ** -53 * 0.1
+
+
+@pytest.mark.parametrize("recon", ["char", "comp"])
+@pytest.mark.parametrize("kind", ["rough", "graded", "wave"])
+def test_small_transverse_velocity(kind, recon):
+    """A transverse velocity of 1e-3 carried by a uniform flow near the speed of
+    sound, constant along y so that no pressure enters its momentum: accurate to
+    its own size.  Bar of one update as above with dt u/dx <= 0.15."""
+    case = wl.smooth_random(2, [331, 61], "spm", seed=5, recon=recon, amp=0.0)
+    rng = np.random.default_rng(8)
+    x = np.arange(331)
+    v = {"rough": rng.standard_normal(331), "graded": 1.0 + 0.2 * rng.uniform(0, 1, 331) ** 4 * rng.standard_normal(331),
+         "wave": np.sin(2 * np.pi * (x + 0.37) / 331)}[kind]
+    W = case["W"].copy()
+    W[0], W[1], W[2], W[3] = 1.0, 1.0, 1e-3 * v, 1.0
+    c = oracle_config(dict(case, W=W))
+    U = oracle.prim_to_cons(c, W)
+    dt = oracle.dt(c, U)
+    ref, _ = oracle.rhs(c, U, 0.5 * dt)
+    s = jxf.Solver(dict(case, W=W), "fp64")
+    R = s.rhs(torch.from_numpy(U).cuda(), 0.5 * dt).cpu().numpy()
+    s.close()
+    err = rhs_update_err(R, ref, U, dt)
+    print(kind, recon, err)
+    assert err[2] < 8 * 2 * 2 * 2.0 ** -53 * 0.15
