@@ -1658,8 +1658,9 @@ __device__ __forceinline__ void reconstruct_w(const Dev &P, const T (&S)[6][MAXV
             const T *w = S[j];
             T val;
             if (v < NP) val = fma(-ent[v], w[IE], w[v]);
-            else if (v == IE) val = fma(h_c, w[in], h_rc2 * w[IE]);
-            else if (v == in) val = fma(-h_c, w[in], h_rc2 * w[IE]);
+            // the larger product (rho c^2 scale) unrounded
+            else if (v == IE) val = fma(h_rc2, w[IE], h_c * w[in]);
+            else if (v == in) val = fma(h_rc2, w[IE], -(h_c * w[in]));
             else val = w[v];
             q[j] = val;
         }
@@ -1715,11 +1716,11 @@ __device__ __forceinline__ void reconstruct_lanes(const Dev &P, const double (&S
 #pragma unroll
         for (int u = 0; u < NP; ++u) ent[u] = Wb[u] * irc2;
         const bool ac = v == in || v == IE, part = v < NP;
-        const double a = part ? -(v == 0 ? ent[0] : ent[NP - 1]) : (v == in ? -h_c : h_c);
+        const double a = part ? -(v == 0 ? ent[0] : ent[NP - 1]) : h_rc2, b = v == in ? -h_c : h_c;
 #pragma unroll
         for (int j = 0; j < 6; ++j) {
-            const double x = ac ? h_rc2 * S[j][IE] : mine(S[j]), y = part ? S[j][IE] : S[j][in];
-            q[j] = ac || part ? fma(a, y, x) : x;
+            const double x = ac ? b * S[j][in] : mine(S[j]);
+            q[j] = ac || part ? fma(a, S[j][IE], x) : x;
         }
     } else {
 #pragma unroll
