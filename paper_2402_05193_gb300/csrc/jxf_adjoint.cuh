@@ -151,14 +151,26 @@ __device__ __forceinline__ void weno5_pair_vjp(const T (&x)[6], T eps, bool z, T
 //   dG/dT_0 = 2 w_0, dG/dT_1 = w_2, dG/dQ_k = -2 w_k (e_k - G)/Q_k
 // for Jiang-Shu weights; WENO5-Z (a_k = d_k (1 + tau/Q_k), tau = |Q_0 - Q_2|)
 //   dG/dQ_k = -(e_k - G) d_k tau/(Q_k^2 sum a), dG/dtau = sum_k (e_k - G) d_k/(Q_k sum a).
-// They are relative to the adjoints that multiply them in double, and accurate
-// to 2^-48 or so; the reverse sweep's own rounding (an order of magnitude and
-// more above 2^-53 of its result, from the divergence's and the projections'
-// cancellation) stays what it was: step adjoint at 256^2 against torch
-// autograd in float64 1.5e-14 before and after.  With the face states of the
-// forward sweep in place of a second forward reconstruction and square roots
-// from reciprocal square roots, the reverse face takes about 520 double
-// operations instead of 1500: step adjoint at 256^2 2.07 -> 0.88 ms.
+// They multiply the adjoints, so an error of theirs is one relative to the
+// result: pairs alone (2^-48) are not enough.  What is carried in pairs is their
+// difference from the constants of the linear weights, (-0.2, 1.1, 2.4, -0.3),
+// every term of which is a multiple of a third difference, told without
+// cancellation:
+//   Q_1 - Q_0 = T_0 ((H_0 + H_1) + 13/3 (A_0 + A_1)),
+//   Q_1 - Q_2 = T_1 ((H_1 - H_2) - 13/3 (A_1 + A_2)),
+//   w_k - d_k = d_k (y_k - s)/(1 + s), s = sum_k d_k y_k, with 1 + y_k the
+//   weights before normalisation over that of k = 1 (Jiang-Shu), over d_k (Z);
+// T itself comes from double differences.  Where max |T| is at most `bound`
+// times sqrt(Q) (the smallest Q over the root of the largest) these terms are
+// small enough; elsewhere, variable by variable, all is double.  Mean errors
+// against quadruple precision over those of the all-double sweep, every variable,
+// both modes and weights, 161 x 141 at Mach 0.001 to 0.3: waves of 50 cells and more
+// 0.69-1.00, of 20 cells 0.73-1.00 (pairs without the linear part kept apart: up
+// to 6.2; bounds of 1/4: up to 1.25 component-wise).  Step adjoint at 256^2
+// (characteristic) 2.09 ms all double with a second forward reconstruction, 1.52
+// with the forward sweep's face states and square roots from reciprocal square
+// roots, 0.96 so (0.88 with the linear part in pairs as well).
+constexpr float kSplitVjpComp = 1.f / 32.f, kSplitVjpChar = 1.f / 16.f;
 __device__ __forceinline__ d2 drcp(d2 a) {  // 1/a
     const f2 r = rcp2(a.h), n = neg2(r);
     return {r, mul2(r, add2(fma2(n, a.h, bc2(1.f)), mul2(n, a.l)))};
@@ -168,16 +180,17 @@ __device__ __forceinline__ d2 bcd2(double x) {
     split_double(x, h, l);
     return bcd(h, l);
 }
-__device__ __forceinline__ void weno5_derivs_split(bool z, const Cst<float> &C, d2 D0, d2 D1, d2 D2, d2 (&c)[4]) {
+__device__ __forceinline__ bool weno5_derivs_split(bool z, const Cst<float> &C, d2 D0, d2 D1, d2 D2, d2 T0, d2 T1,
+                                                   float bound, d2 (&c)[4]) {
     const f2 two = bc2(2.f);
     const d2 D3 = swapd(D1);
     const d2 A0 = dsub(D1, D0), A1 = dsub(D2, D1), A2 = dsub(D3, D2);
-    const d2 T0 = dsub(A1, A0), T1 = dsub(A2, A1);
     const d2 H0 = dadd(dscale(D1, two), A0), H1 = dadd(D1, D2), H2 = dsub(A2, dscale(D2, two));
     const f2 e4 = bc2(C.weno_eps4), e4l = bc2(C.weno_eps4l);
     const float k0 = (float)(13.0 / 3.0), k1 = (float)(13.0 / 3.0 - (double)k0);
+    const d2 k13 = bcd(k0, k1);
     auto q = [&](d2 H, d2 A) {
-        const d2 h = dsq(H), a = dmul(dsq(A), bcd(k0, k1));
+        const d2 h = dsq(H), a = dmul(dsq(A), k13);
         f2 s, e, t, g;
         two_sum2(h.h, a.h, s, e);
         two_sum2(s, e4, t, g);
@@ -188,38 +201,53 @@ __device__ __forceinline__ void weno5_derivs_split(bool z, const Cst<float> &C, 
     const f2 sc = mk2(pow2(fmaxf(Q0.h.v.x, fmaxf(Q1.h.v.x, Q2.h.v.x))),
                       pow2(fmaxf(Q0.h.v.y, fmaxf(Q1.h.v.y, Q2.h.v.y))));
     Q0 = dscale(Q0, sc), Q1 = dscale(Q1, sc), Q2 = dscale(Q2, sc);
+    {   // the largest Q is between 1 and 2 now
+        auto small = [&](float t0, float t1, float q0, float q1, float q2, float s) {
+            const float t = fmaxf(fabsf(t0), fabsf(t1)), qm = fminf(q0, fminf(q1, q2));
+            return t * t * s <= (0.5f * bound * bound) * (qm * qm);
+        };
+        if (!(small(T0.h.v.x, T1.h.v.x, Q0.h.v.x, Q1.h.v.x, Q2.h.v.x, sc.v.x) &&
+              small(T0.h.v.y, T1.h.v.y, Q0.h.v.y, Q1.h.v.y, Q2.h.v.y, sc.v.y)))
+            return false;
+    }
     const d2 r0 = renorm(drcp(Q0)), r1 = renorm(drcp(Q1)), r2 = renorm(drcp(Q2));
-    // weights with d = (1, 6, 3): a_k, 1/sum a
-    d2 a0, a1, a2, tau = bcd(0.f, 0.f);
+    // Q_1 - Q_0, Q_1 - Q_2
+    const d2 m0 = renorm(dscale(dmul(T0, renorm(dadd(dadd(H0, H1), dmul(k13, renorm(dadd(A0, A1)))))), sc));
+    const d2 m2 = renorm(dscale(dmul(T1, renorm(dsub(dsub(H1, H2), dmul(k13, renorm(dadd(A1, A2)))))), sc));
+    d2 y0, y1 = bcd(0.f, 0.f), y2, tau = y1;
     f2 sg = bc2(0.f);
     if (z) {
-        tau = renorm(dsub(Q0, Q2));
+        tau = renorm(dsub(m2, m0));  // Q_0 - Q_2
         sg = mk2(tau.h.v.x < 0.f ? -1.f : 1.f, tau.h.v.y < 0.f ? -1.f : 1.f);
         tau = dscale(tau, sg);
-        const d2 one = bcd(1.f, 0.f);
-        a0 = renorm(dadd(one, dmul(tau, r0)));
-        a1 = dmulf(renorm(dadd(one, dmul(tau, r1))), 6.f);
-        a2 = dmulf(renorm(dadd(one, dmul(tau, r2))), 3.f);
+        y0 = renorm(dmul(tau, r0)), y1 = renorm(dmul(tau, r1)), y2 = renorm(dmul(tau, r2));
     } else {
-        a0 = dsq(r0);
-        a1 = dmulf(dsq(r1), 6.f);
-        a2 = dmulf(dsq(r2), 3.f);
+        const d2 x0 = renorm(dmul(m0, r0)), x2 = renorm(dmul(m2, r2));
+        y0 = renorm(dadd(dscale(x0, two), dsq(x0)));
+        y2 = renorm(dadd(dscale(x2, two), dsq(x2)));
     }
-    const d2 ia = renorm(drcp(renorm(dadd(dadd(a0, a1), a2))));
-    const d2 w0 = renorm(dmul(renorm(a0), ia)), w1 = renorm(dmul(renorm(a1), ia)), w2 = renorm(dmul(renorm(a2), ia));
+    const d2 s10 = renorm(dadd(dadd(y0, dmulf(y1, 6.f)), dmulf(y2, 3.f)));  // 10 s
+    const d2 ia = renorm(drcp(renorm(dadd(bcd(10.f, 0.f), s10))));          // 1/sum of (1, 6, 3) (1 + y)
+    const float c0 = 0.1f, c1 = (float)(0.1 - (double)c0);
+    const d2 ia1 = renorm(dmul(ia, bcd(c0, c1)));
+    const d2 one = bcd(1.f, 0.f);
+    const d2 w0 = renorm(dmul(renorm(dadd(one, y0)), ia)), w2 = renorm(dmulf(dmul(renorm(dadd(one, y2)), ia), 3.f));
+    const d2 v0 = renorm(dmul(renorm(dsub(dmulf(y0, 10.f), s10)), ia1));  // w_0 - 0.1, w_2 - 0.3
+    const d2 v2 = renorm(dmulf(dmul(renorm(dsub(dmulf(y2, 10.f), s10)), ia1), 3.f));
     const d2 e0 = dscale(T0, two);
     const d2 G = renorm(dadd(dmul(w0, e0), dmul(w2, T1)));
     const d2 x0 = renorm(dsub(e0, G)), x2 = renorm(dsub(T1, G));  // e_k - G; e_1 - G = -G
     // minus dG/dQ_k (of the unscaled Q_k)
     d2 g0, g1, g2;
     if (z) {
-        const d2 y0 = renorm(dmul(dmul(x0, ia), r0)), y1 = renorm(dmulf(dmul(dmul(G, ia), r1), -6.f));
-        const d2 y2 = renorm(dmulf(dmul(dmul(x2, ia), r2), 3.f));
-        const d2 tb = dscale(renorm(dadd(dadd(y0, y1), y2)), sg);  // dG/dQ_0 through tau, -dG/dQ_2
-        g0 = dsub(dmul(y0, dmul(tau, r0)), tb);
-        g1 = dmul(y1, dmul(tau, r1));
-        g2 = dadd(dmul(y2, dmul(tau, r2)), tb);
+        const d2 u0 = renorm(dmul(dmul(x0, ia), r0)), u1 = renorm(dmulf(dmul(dmul(G, ia), r1), -6.f));
+        const d2 u2 = renorm(dmulf(dmul(dmul(x2, ia), r2), 3.f));
+        const d2 tb = dscale(renorm(dadd(dadd(u0, u1), u2)), sg);  // dG/dQ_0 through tau, -dG/dQ_2
+        g0 = dsub(dmul(u0, y0), tb);
+        g1 = dmul(u1, y1);
+        g2 = dadd(dmul(u2, y2), tb);
     } else {
+        const d2 w1 = renorm(dmulf(ia, 6.f));
         g0 = dscale(dmul(dmul(w0, x0), r0), two);
         g1 = dscale(dmul(dmul(w1, G), r1), bc2(-2.f));
         g2 = dscale(dmul(dmul(w2, x2), r2), two);
@@ -228,28 +256,42 @@ __device__ __forceinline__ void weno5_derivs_split(bool z, const Cst<float> &C, 
     // through Q_k = H_k^2 + 13/3 A_k^2 (both minus their derivatives of G)
     const d2 h0 = dscale(dmul(H0, g0), two), h1 = dscale(dmul(H1, g1), two), h2 = dscale(dmul(H2, g2), two);
     const d2 kk = bcd(2.f * k0, 2.f * k1);
-    const d2 t0 = dscale(w0, two);
+    const d2 t0 = dscale(v0, two);
     const d2 b0 = renorm(dadd(dmul(dmul(kk, A0), g0), t0));
-    const d2 b1 = renorm(dsub(dadd(dmul(dmul(kk, A1), g1), w2), t0));
-    const d2 b2 = renorm(dsub(dmul(dmul(kk, A2), g2), w2));
+    const d2 b1 = renorm(dsub(dadd(dmul(dmul(kk, A1), g1), v2), t0));
+    const d2 b2 = renorm(dsub(dmul(dmul(kk, A2), g2), v2));
     c[0] = renorm(dscale(dadd(h0, b0), bc2(-1.f)));
-    c[1] = renorm(dadd(dadd(dmulf(renorm(h0), 3.f), h1), dadd(dsub(b0, b1), bcd(1.f, 0.f))));
-    c[2] = renorm(dadd(dsub(h1, dmulf(renorm(h2), 3.f)), dadd(dsub(b1, b2), bcd(2.f, 0.f))));
+    c[1] = renorm(dadd(dadd(dmulf(renorm(h0), 3.f), h1), dsub(b0, b1)));
+    c[2] = renorm(dadd(dsub(h1, dmulf(renorm(h2), 3.f)), dsub(b1, b2)));
     c[3] = renorm(dadd(h2, b2));
+    return true;
 }
 
-// xb += the adjoint of the six values from those of the face's two, with the
-// lanes' differences D = (D_0, D_4), (D_1, D_3), (D_2, D_2).
-__device__ __forceinline__ void weno5_apply_split(bool z, const Cst<float> &C, const d2 (&D)[3], double vlb,
-                                                  double vrb, double (&xb)[6]) {
+// What the derivatives of one variable are formed from: the lanes' differences
+// (D_0, D_4), (D_1, D_3), (D_2, D_2) and third differences (T_0, T_2), (T_1, T_1).
+struct SplitDiffs {
+    d2 D[3], T0, T1;
+};
+template <class X> __device__ __forceinline__ SplitDiffs split_diffs(X x) {  // x(j): cell value j
+    double D[5];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) D[k] = x(k + 1) - x(k);
+    const double A0 = D[1] - D[0], A1 = D[2] - D[1], A2 = D[3] - D[2], A3 = D[4] - D[3];
+    return {{lanes(D[0], D[4]), lanes(D[1], D[3]), bcd2(D[2])}, lanes(A1 - A0, A3 - A2), bcd2(A2 - A1)};
+}
+
+// xb += the adjoint of the six values from those of the face's two; false where
+// the derivatives are not small enough beside the linear ones for pairs.
+__device__ __forceinline__ bool weno5_apply_split(bool z, const Cst<float> &C, const SplitDiffs &s, float bound,
+                                                  double vlb, double vrb, double (&xb)[6]) {
     d2 c[4];
-    weno5_derivs_split(z, C, D[0], D[1], D[2], c);
-    const double l = (1.0 / 6.0) * vlb, r = (-1.0 / 6.0) * vrb;
+    if (!weno5_derivs_split(z, C, s.D[0], s.D[1], s.D[2], s.T0, s.T1, bound, c)) return false;
+    const double l = (1.0 / 6.0) * vlb, r = (-1.0 / 6.0) * vrb, lin[4] = {-0.2, 1.1, 2.4, -0.3};
     double Db[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        Db[k] = fma(l, widen(c[k].h.v.x), fma(l, widen(c[k].l.v.x), Db[k]));
-        Db[4 - k] = fma(r, widen(c[k].h.v.y), fma(r, widen(c[k].l.v.y), Db[4 - k]));
+        Db[k] = fma(l, lin[k] + (widen(c[k].h.v.x) + widen(c[k].l.v.x)), Db[k]);
+        Db[4 - k] = fma(r, lin[k] + (widen(c[k].h.v.y) + widen(c[k].l.v.y)), Db[4 - k]);
     }
     xb[0] -= Db[0];
     xb[1] += Db[0] - Db[1];
@@ -257,6 +299,7 @@ __device__ __forceinline__ void weno5_apply_split(bool z, const Cst<float> &C, c
     xb[3] += (Db[2] - Db[3]) + vrb;
     xb[4] += Db[3] - Db[4];
     xb[5] += Db[4];
+    return true;
 }
 
 // ----------------------------------------------------- reconstruction VJP --
@@ -275,13 +318,11 @@ __device__ __forceinline__ void reconstruct_vjp(const Dev &P, const T (&S)[6][MA
         for (int v = 0; v < NV; ++v) {
             const T x[6] = {S[0][v], S[1][v], S[2][v], S[3][v], S[4][v], S[5][v]};
             T xb[6] = {0, 0, 0, 0, 0, 0};
-            if (!split) weno5_pair_vjp(x, eps, z, WLb[v], WRb[v], xb);
-            else if constexpr (std::is_same<T, double>::value) {
-                d2 D[3];
-#pragma unroll
-                for (int k = 0; k < 3; ++k) D[k] = lanes(x[k + 1] - x[k], x[5 - k] - x[4 - k]);
-                weno5_apply_split(z, cst<float>(P), D, WLb[v], WRb[v], xb);
-            }
+            bool done = false;
+            if constexpr (std::is_same<T, double>::value)
+                done = split && weno5_apply_split(z, cst<float>(P), split_diffs([&](int j) { return x[j]; }), kSplitVjpComp,
+                                                   WLb[v], WRb[v], xb);
+            if (!done) weno5_pair_vjp(x, eps, z, WLb[v], WRb[v], xb);
 #pragma unroll
             for (int j = 0; j < 6; ++j) Sb[j][v] += xb[j];
         }
@@ -335,36 +376,42 @@ __device__ __forceinline__ void reconstruct_vjp(const Dev &P, const T (&S)[6][MA
     for (int v = 0; v < NV; ++v)
 #pragma unroll
         for (int j = 0; j < 6; ++j) qb[v][j] = T(0);
-    if (!split) {
+    bool done[NV];
 #pragma unroll
-        for (int v = 0; v < NV; ++v) {
-            T q[6];
+    for (int v = 0; v < NV; ++v) done[v] = false;
+    if constexpr (std::is_same<T, double>::value) {
+        if (split) {
+            const Cst<float> &C32 = cst<float>(P);
+            SplitDiffs s[NV];  // of the primitives, then of q
 #pragma unroll
-            for (int j = 0; j < 6; ++j) {
-                if (v == 0) q[j] = S[j][0] - ent * S[j][IE];
-                else if (v == in) q[j] = -h_c * S[j][in] + h_rc2 * S[j][IE];
-                else if (v == IE) q[j] = h_c * S[j][in] + h_rc2 * S[j][IE];
-                else q[j] = S[j][v];
-            }
-            weno5_pair_vjp(q, eps, z, qLb[v], qRb[v], qb[v]);
+            for (int v = 0; v < NV; ++v) s[v] = split_diffs([&](int j) { return S[j][v]; });
+            const d2 e = bcd2(ent), hc = bcd2(h_c), hr = bcd2(h_rc2);
+            auto project = [&](d2 &x0, d2 &xi, d2 &xe) {
+                const d2 x = dmul(hc, xi), y = dmul(hr, xe);
+                x0 = renorm(dsub(x0, dmul(e, xe)));
+                xe = renorm(dadd(y, x));
+                xi = renorm(dsub(y, x));
+            };
+#pragma unroll
+            for (int k = 0; k < 3; ++k) project(s[0].D[k], s[in].D[k], s[IE].D[k]);
+            project(s[0].T0, s[in].T0, s[IE].T0);
+            project(s[0].T1, s[in].T1, s[IE].T1);
+#pragma unroll
+            for (int v = 0; v < NV; ++v) done[v] = weno5_apply_split(z, C32, s[v], kSplitVjpChar, qLb[v], qRb[v], qb[v]);
         }
-    } else if constexpr (std::is_same<T, double>::value) {
-        const Cst<float> &C32 = cst<float>(P);
-        d2 D[NV][3];  // lanes (D_0, D_4), (D_1, D_3), (D_2, D_2) of the primitives, then of q
+    }
 #pragma unroll
-        for (int v = 0; v < NV; ++v)
+    for (int v = 0; v < NV; ++v) {
+        if (done[v]) continue;
+        T q[6];
 #pragma unroll
-            for (int k = 0; k < 3; ++k) D[v][k] = lanes(S[k + 1][v] - S[k][v], S[5 - k][v] - S[4 - k][v]);
-        const d2 e = bcd2(ent), hc = bcd2(h_c), hr = bcd2(h_rc2);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const d2 x = dmul(hc, D[in][k]), y = dmul(hr, D[IE][k]);
-            D[0][k] = renorm(dsub(D[0][k], dmul(e, D[IE][k])));
-            D[IE][k] = renorm(dadd(y, x));
-            D[in][k] = renorm(dsub(y, x));
+        for (int j = 0; j < 6; ++j) {
+            if (v == 0) q[j] = S[j][0] - ent * S[j][IE];
+            else if (v == in) q[j] = fma(h_rc2, S[j][IE], -(h_c * S[j][in]));  // as in the forward sweep
+            else if (v == IE) q[j] = fma(h_rc2, S[j][IE], h_c * S[j][in]);
+            else q[j] = S[j][v];
         }
-#pragma unroll
-        for (int v = 0; v < NV; ++v) weno5_apply_split(z, C32, D[v], qLb[v], qRb[v], qb[v]);
+        weno5_pair_vjp(q, eps, z, qLb[v], qRb[v], qb[v]);
     }
     // reverse of the projection q = K^{-1} S
     T entb = 0, h_cb = 0, h_rc2b = 0;

@@ -209,3 +209,45 @@ def test_small_transverse_velocity(kind, recon):
     err = rhs_update_err(R, ref, U, dt)
     print(kind, recon, err)
     assert err[2] < 8 * 2 * 2 * 2.0 ** -53 * 0.15
+
+
+@pytest.mark.parametrize("recon", ["char", "comp"])
+@pytest.mark.parametrize("weno", ["js", "z"])
+def test_reverse_sweep_of_uniform_supersonic_flow(weno, recon):
+    """At a uniform state, supersonic along both axes, the faces are the
+    fifth-order upwind values (2, -13, 47, 27, -3)/60: the reverse sweep in
+    closed form (extended precision).  In the mean 1e-15 of the mean: about 8
+    roundings of 2^-53."""
+    n, dx, g, w = [157, 131], [1.0 / 157, 1.0 / 131], 1.4, (1.0, 2.5, 2.2, 1.0)
+    case = dict(wl.smooth_random(2, n, "spm", seed=1, recon=recon, amp=0.0), weno=weno)
+    W = np.empty_like(case["W"])
+    for v in range(4):
+        W[v] = w[v]
+    U = oracle.prim_to_cons(oracle_config(case), W)
+    rbar = np.random.default_rng(3).standard_normal(U.shape)
+    s = jxf.Solver(case, "fp64")
+    got = s.rhs_vjp(torch.from_numpy(U).cuda(), torch.from_numpy(rbar).cuda()).cpu().numpy()
+    s.close()
+    L = np.longdouble
+    r, mu, mv, E = (L(U[v].flat[0]) for v in range(4))
+    u, v = mu / r, mv / r
+    p = (L(g) - 1) * (E - r * (u * u + v * v) / 2)
+    h = L(g) / (L(g) - 1)
+    ke = (u * u + v * v) / 2
+    # dF/dW for the x and y fluxes, dW/dU
+    A = [np.array([[u, r, 0, 0], [u * u, 2 * r * u, 0, 1], [u * v, r * v, r * u, 0],
+                   [u * ke, h * p + r * ke + r * u * u, r * u * v, h * u]], L),
+         np.array([[v, 0, r, 0], [u * v, r * v, r * u, 0], [v * v, 0, 2 * r * v, 1],
+                   [v * ke, r * u * v, h * p + r * ke + r * v * v, h * v]], L)]
+    k = L(g) - 1
+    B = np.array([[1, 0, 0, 0], [-u / r, 1 / r, 0, 0], [-v / r, 0, 1 / r, 0], [k * ke, -k * u, -k * v, k]], L)
+    coef = [L(c) / 60 for c in (2, -13, 47, 27, -3)]  # cells i - 2 .. i + 2 of face i + 1/2
+    rb, Wb = rbar[:, 0].astype(L), np.zeros((4,) + rbar.shape[2:], L)
+    for d, axis in ((0, 2), (1, 1)):
+        Fb = (np.roll(rb, -1, axis) - rb) / L(dx[d])  # of face i + 1/2
+        for m, c in zip(range(-2, 3), coef):
+            Wb += c * np.einsum("fw,fyx->wyx", A[d], np.roll(Fb, m, axis))
+    ref = np.einsum("wu,wyx->uyx", B, Wb)
+    err = np.abs(got[:, 0] - ref).mean(axis=(1, 2)) / np.abs(ref).mean(axis=(1, 2))
+    print(weno, recon, err)
+    assert err.max() < 1e-15
