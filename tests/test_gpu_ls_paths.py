@@ -122,3 +122,64 @@ def test_extension_leaves_out_empty_blocks(ndim, n, centre):
     jxf.jxf_ls_extend(grid, d, al, dg, nr, want, ndim + 1, 2, 20, z(ndim + 1))
     assert want.abs().max() > 0.1
     assert (got - want).abs().max() < 1e-13 * want.abs().max()
+
+
+def _same_with_nans(a, b):
+    a, b = a.cpu().numpy(), b.cpu().numpy()
+    assert np.isnan(b).any() and np.array_equal(np.isnan(a), np.isnan(b))
+    assert np.abs(np.nan_to_num(a) - np.nan_to_num(b)).max() < 1e-13
+
+
+@pytest.mark.parametrize("steps", [1, 4, 20])
+def test_extension_with_a_nan_normal(steps):
+    """A NaN normal component in a cell whose values and neighbours are +0: 0
+    times NaN is evaluated.  Against the same data with 1e-290 for 0, where
+    nothing is left out."""
+    n, h, bc = [23, 19, 17], 1.0 / 16, [(P, P), (Z, S), (S, Z)]
+    cfg, grid = orc.ls_config(ndim=3, n=n, h=h, bc=bc), jxf.ls_grid(3, n, h, bc)
+    phi = _phi(3, n, h, 3, 0.05)
+    _, al, dg, nr = orc.ls_geometry(cfg, phi)
+    cut = ((al > 0) & (al < 1)) | (dg > 0)
+    k = tuple(np.argwhere(~cut & (np.abs(phi) > 3.5 * h))[0])
+    nr[(0,) + k] = np.nan
+    out = []
+    for zero in (0.0, 1e-290):
+        q = np.where(cut, np.random.default_rng(4).uniform(-1, 1, (4,) + phi.shape), zero)
+        d = [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in (phi, al, dg, nr, q)]
+        jxf.jxf_ls_extend(grid, *d, 4, 2, steps, torch.empty(4 * phi.size, dtype=torch.float64, device="cuda"))
+        out.append(d[4])
+    _same_with_nans(*out)
+
+
+@pytest.mark.parametrize("ndim,n,bad", [(2, [50, 40], (30, 25)), (2, [256, 9], (4, 100)), (3, [24, 21, 18], (9, 12, 12))])
+def test_empty_blocks_beside_a_nan(ndim, n, bad):
+    """A NaN level set in an otherwise empty block: the interface quantities of
+    jxf_ls_init, which leave empty blocks out, are NaN where the plain
+    extension's are."""
+    h, bc, gamma, pinf = 1.0 / 16, [(P, P)] * ndim, (1.4, 1.67), (0.0, 0.3)
+    grid = jxf.ls_grid(ndim, n, h, bc)
+    mesh = np.meshgrid(*[(np.arange(m) - 4.3) * h for m in n][::-1], indexing="ij")
+    phi = 1.6 * h - np.sqrt(sum(m * m for m in mesh))
+    phi[tuple(min(b, s - 1) for b, s in zip(bad, phi.shape))] = np.nan
+    rng = np.random.default_rng(5)
+    W = [torch.from_numpy(rng.uniform(0.5, 1.5, (ndim + 2,) + phi.shape)).cuda() for _ in range(2)]
+    eos = []
+    for k in range(2):
+        e = jxf.jxf_eos()
+        e.model = jxf.JXF_SPM
+        e.gamma[0] = e.gamma[1] = gamma[k]
+        e.pinf[0] = e.pinf[1] = pinf[k]
+        eos.append(e)
+    sch = jxf.jxf_scheme()
+    sch.recon, sch.precision, sch.weno_eps = jxf.JXF_WENO5JS_CHAR, jxf.JXF_FP64, 1e-6
+    d = torch.from_numpy(np.ascontiguousarray(phi)).cuda()
+    z = lambda k: torch.zeros((k,) + phi.shape, dtype=torch.float64, device="cuda")
+    got = z(ndim + 1)
+    work = torch.full((jxf.jxf_ls_step_work(grid),), 3.0, dtype=torch.float64, device="cuda")
+    jxf.jxf_ls_init(grid, *eos, sch, d, *W, z(ndim + 2), z(ndim + 2), got, work)
+    ap = torch.zeros(jxf.jxf_ls_nface(grid), dtype=torch.float64, device="cuda")
+    al, dg, nr, want = z(1)[0], z(1)[0], z(ndim), z(ndim + 1)
+    jxf.jxf_ls_geometry(grid, d, ap, al, dg, nr)
+    jxf.jxf_ls_interface(grid, *W, gamma, pinf, al, dg, nr, want[:ndim], want[ndim])
+    jxf.jxf_ls_extend(grid, d, al, dg, nr, want, ndim + 1, 2, 20, z(ndim + 1))
+    _same_with_nans(got, want)
