@@ -32,6 +32,10 @@ namespace jxf {
 
 constexpr int MAXV = 7;
 constexpr int kFluxThreads = 128;
+// Streaming multiprocessors of the GB300 this library is built for (four FP64
+// pipes each).  A constant, not the device's count: with kSplitFaces it decides
+// which arithmetic a face takes, and results are not to depend on the device.
+constexpr int kSMs = 152;
 // minimum resident blocks of the face sweep per SM (register budget), per
 // storage type (double: see the split weights below); overridable at build time for tuning sweeps
 #ifndef JXF_FLUX_MINB64
@@ -1038,7 +1042,7 @@ __device__ __forceinline__ float high_float(unsigned a) {
     return a < 0x38100000u ? 0.f : __uint_as_float(((a << 3) ^ 0x40000000u) & 0x7FFFFFFFu);
 }
 
-constexpr long long kSplitFaces = 4 * 152 * 32 + 1;
+constexpr long long kSplitFaces = 4 * kSMs * 32 + 1;
 constexpr float kSplitD = 1.f / 16.f;   // bound of |D| over the variable's scale
 constexpr float kSplitT = 1.f / 128.f;  // bound of |T|
 constexpr float kSplitOwn = 1.f / 16.f;  // bound of a transverse velocity's |T| over its largest value

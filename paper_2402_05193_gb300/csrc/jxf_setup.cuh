@@ -123,7 +123,7 @@ inline void fill_dev(const jxf_grid *grid, const jxf_eos *eos, const jxf_scheme 
     // an SM, and every warp an FP64 pipe, to itself
     const int group = eos->model == JXF_DIM ? kLaneGroup<5> : kLaneGroup<3>;
     P.line_group = grid->ndim == 1 && f64 && !P.teno &&
-                           grid->n[0] <= 152 * (kFluxThreads / group - 1)
+                           grid->n[0] <= kSMs * (kFluxThreads / group - 1)
                        ? group
                        : 1;
     P.eps_rho = scheme->eps_rho > 0.0 ? scheme->eps_rho : (f64 ? 1e-12 : 1e-10);
