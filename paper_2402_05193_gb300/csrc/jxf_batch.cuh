@@ -78,13 +78,9 @@ __global__ void __launch_bounds__(kFluxThreads, SweepMinBlocks<T, RSV>::value)
 }
 
 // Cell tiles hold at most one block of cells; with epi the tile's partials
-// go to its slot.  Five blocks per SM in float (48 registers): at the eight of
-// the other cell kernels (32) the five-equation update spills 108 bytes a
-// thread beside the tile loop.  96 drops, stage 1 | 2 | 3: 119 | 130 | 140 us at
-// eight, 116 | 118 | 131 at six, 109 | 114 | 126 at five, 115 | 118 | 134 at four.
-template <typename T> constexpr int kUpdateBatchBlocks = sizeof(T) == 4 ? 5 : CellMinBlocks<T>::value;
+// go to its slot.
 template <typename T, int MODEL, int NDIM>
-__global__ void __launch_bounds__(kCellThreads, kUpdateBatchBlocks<T>)
+__global__ void __launch_bounds__(kCellThreads, kUpdateMinBlocks<T>)
     k_update_batch(const Dev *__restrict__ devs, const Tile *__restrict__ tiles, int ntiles,
                    unsigned *ticket, double *part, int epi) {
     using V = Vars<MODEL, NDIM>;

@@ -64,6 +64,13 @@ constexpr int kCellThreads = 256;
 #endif
 template <typename T> struct CellMinBlocks { static constexpr int value = JXF_CELL_MINB32; };
 template <> struct CellMinBlocks<double> { static constexpr int value = JXF_CELL_MINB64; };
+// The update kernels (k_update, k_update_batch) in float: five blocks per SM (48
+// registers).  At eight (32) the face values are loaded a few at a time, and the
+// five-equation batch update spills 108 bytes a thread beside the tile loop.  us:
+// right-hand side 18x14x16 viscous 54.7 at eight, 52.4 at five, five-equation
+// 128x64x64 132.6, 129.6; batch of 96 drops, stage 1 | 2 | 3: 119 | 130 | 140 at eight,
+// 116 | 118 | 131 at six, 109 | 114 | 126 at five, 115 | 118 | 134 at four.
+template <typename T> constexpr int kUpdateMinBlocks = sizeof(T) == 4 ? 5 : CellMinBlocks<T>::value;
 
 // device scalar slots (double)
 enum {
@@ -3281,7 +3288,7 @@ template <typename T> __device__ __forceinline__ T block_cdt(const Dev &P, doubl
 }
 
 template <typename T, int MODEL, int NDIM>
-__global__ void __launch_bounds__(kCellThreads, CellMinBlocks<T>::value)
+__global__ void __launch_bounds__(kCellThreads, kUpdateMinBlocks<T>)
     k_update(const Dev P, const int mode, const int epi) {
     using V = Vars<MODEL, NDIM>;
     constexpr int NV = V::NV;
