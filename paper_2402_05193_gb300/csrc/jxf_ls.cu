@@ -419,29 +419,41 @@ __device__ __forceinline__ double weno3(double v1, double v2, double v3, double 
     return q1 + jxf::fdiv(s1 * (q0 - q1), s1 + 2.0 * s0);
 }
 
+// The cells a cell's derivatives are formed from: itself and two on each side
+// along every axis (x[d][0..3]: -2, -1, 1, 2).
+template <int NDIM> struct ReinitCells {
+    double x0, x[NDIM][4];
+    __device__ __forceinline__ ReinitCells(const LsGrid &g, const double *__restrict__ p, const int (&c)[3], long long i) {
+        x0 = __ldg(p + i);
+#pragma unroll
+        for (int d = 0; d < NDIM; ++d)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) x[d][k] = ls_line(g, p, i, c[d], d, k < 2 ? k - 2 : k - 1);
+    }
+};
+
 // R_reinit = -sgn(phi0) (|grad phi| - 1) with the Godunov Hamiltonian of the
 // one-sided derivatives, 0 where |R| <= thr.  need: bit d (d + 3) set where
 // the left (right) derivative of axis d may enter; the others would be cut to
 // 0 by their sign.
 template <int NDIM>
-__device__ __forceinline__ double reinit_r(const LsGrid &g, const double *__restrict__ p, double phi0, double thr,
-                                           const int (&c)[3], long long i, unsigned need) {
+__device__ __forceinline__ double reinit_r(const LsGrid &g, const ReinitCells<NDIM> &p, double phi0, double thr,
+                                           unsigned need) {
     const bool spos = ls_pos(phi0);
     const double s = spos ? 1.0 : (ls_neg(phi0) ? -1.0 : 0.0);
     const double eps = 1e-6 * g.h * g.h;
     double h2 = 0.0;
 #pragma unroll
     for (int d = 0; d < NDIM; ++d) {
-        const double pm1 = ls_line(g, p, i, c[d], d, -1), p0 = __ldg(p + i), pp1 = ls_line(g, p, i, c[d], d, 1);
-        const double dm = p0 - pm1, dp = pp1 - p0;
+        const double dm = p.x0 - p.x[d][1], dp = p.x[d][2] - p.x0;
         double q1 = 0.0, q2 = 0.0;
         if ((need >> d) & 1u) {
-            const double a = weno3(pm1 - ls_line(g, p, i, c[d], d, -2), dm, dp, eps) * g.ih;
+            const double a = weno3(p.x[d][1] - p.x[d][0], dm, dp, eps) * g.ih;
             const double t1 = (spos ? ls_pos(a) : ls_neg(a)) ? a : 0.0;
             q1 = t1 * t1;
         }
         if ((need >> (d + 3)) & 1u) {
-            const double b = weno3(ls_line(g, p, i, c[d], d, 2) - pp1, dp, dm, eps) * g.ih;
+            const double b = weno3(p.x[d][3] - p.x[d][2], dp, dm, eps) * g.ih;
             const double t2 = (spos ? ls_neg(b) : ls_pos(b)) ? b : 0.0;
             q2 = t2 * t2;
         }
@@ -470,11 +482,10 @@ __device__ __forceinline__ float ls_trunc(double x) {
 // axes does by sqrt(3).  64 e covers this and the float evaluation's own
 // rounding (below 2^-18 of a derivative) with a factor of five to spare.
 template <int NDIM>
-__device__ __forceinline__ bool reinit_screen(const LsGrid &g, const double *__restrict__ p, double phi0, float thr,
-                                              const int (&c)[3], long long i, unsigned &need) {
-    const double pc = __ldg(p + i);
-    const float ih = (float)g.ih, f0 = ls_trunc(pc);
-    unsigned top = max(ls_top(pc), ls_top(phi0));
+__device__ __forceinline__ bool reinit_screen(const LsGrid &g, const ReinitCells<NDIM> &p, double phi0, float thr,
+                                              unsigned &need) {
+    const float ih = (float)g.ih, f0 = ls_trunc(p.x0);
+    unsigned top = max(ls_top(p.x0), ls_top(phi0));
     float v[NDIM][4];  // D_{-2}, D_{-1}, D_0, D_1 of each axis over h
     float m = fabsf(f0), D = 0.f;
 #pragma unroll
@@ -482,9 +493,8 @@ __device__ __forceinline__ bool reinit_screen(const LsGrid &g, const double *__r
         float f[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const double x = ls_line(g, p, i, c[d], d, k < 2 ? k - 2 : k - 1);
-            top = max(top, ls_top(x));
-            f[k] = ls_trunc(x);
+            top = max(top, ls_top(p.x[d][k]));
+            f[k] = ls_trunc(p.x[d][k]);
             m = fmaxf(m, fabsf(f[k]));
         }
         v[d][0] = (f[1] - f[0]) * ih;
@@ -526,44 +536,61 @@ __device__ __forceinline__ bool reinit_screen(const LsGrid &g, const double *__r
 // gathered and evaluated in double, without the one-sided derivatives whose
 // sign is certain to cut them.  The results are those of evaluating every cell
 // in double.  Bound by the FP64 pipe (150 operations a cell before, all
-// cells); 246 -> 41 us per stage on a 96^3 drop whose distance function is
-// distorted by 3 %.
-template <int NDIM>
+// cells); 246 -> 23 us for R on 96^3 cells near a distance function.
+// Grids of at most one block per SM are bound by one warp's latency instead: no
+// gathering there, each lane goes on with the cells it has loaded.  us for 10
+// pseudo-time steps, all cells near a distance function | a quarter of them not |
+// none, all in double / ungathered / gathered: 32^3 299 / 133 | 285 | 341 / 146 | 292 |
+// 375; 40^3 504 / 146 | 437 | 546 / 156 | 368 | 582; 96^3 4934 / 443 | 1601 | 4181 / 443
+// | 1487 | 4304.  (Far from a distance function everywhere the screen is lost
+// time: on grids below 48^3 the all-double kernel was faster by up to 16 %.)
+constexpr long long kReinitGather = (long long)jxf::kSMs * kLsThreads;
+template <int NDIM, bool GATHER>
 __global__ void __launch_bounds__(kLsThreads) k_ls_reinit(const LsGrid g, const double *__restrict__ ps,
                                                          const double *pn, const double *__restrict__ p0, double thr,
                                                          float thr_lo, double dtau, int mode, double *out) {
-    __shared__ unsigned list[kLsThreads];
+    __shared__ unsigned list[GATHER ? kLsThreads : 1];
     __shared__ int count;
-    if (threadIdx.x == 0) count = 0;
-    __syncthreads();
+    if constexpr (GATHER) {
+        if (threadIdx.x == 0) count = 0;
+        __syncthreads();
+    }
     const long long i0 = (long long)blockIdx.x * blockDim.x, i = i0 + threadIdx.x;
+    auto put = [&](long long j, double r) {
+        if (mode < 0) out[j] = r;
+        else if (mode == 0) out[j] = ps[j] + dtau * r;
+        else out[j] = 0.5 * pn[j] + 0.5 * (ps[j] + dtau * r);
+    };
     bool full = false;
     unsigned need = 0;
     if (i < g.ncell) {
         int c[3];
         ls_cell(g, i, c);
-        full = !reinit_screen<NDIM>(g, ps, __ldg(p0 + i), thr_lo, c, i, need);
+        const ReinitCells<NDIM> x(g, ps, c, i);
+        const double phi0 = __ldg(p0 + i);
+        full = !reinit_screen<NDIM>(g, x, phi0, thr_lo, need);
         if (!full) {  // R = 0
-            const double q = __ldg(ps + i) , z = __double_as_longlong(q) << 1 ? q : 0.0;  // -0 + 0 = 0
+            const double q = x.x0, z = __double_as_longlong(q) << 1 ? q : 0.0;  // -0 + 0 = 0
             if (mode < 0) out[i] = 0.0;
             else if (mode == 0) out[i] = z;
             else {
                 const double o = pn[i];
                 out[i] = __double_as_longlong(o) == __double_as_longlong(z) ? z : 0.5 * o + 0.5 * z;
             }
+        } else if constexpr (!GATHER) {
+            put(i, reinit_r<NDIM>(g, x, phi0, thr, need));
         }
     }
-    ls_gather(full, threadIdx.x | (need << 16), list, &count);
-    __syncthreads();
-    for (int t = threadIdx.x; t < count; t += kLsThreads) {
-        const unsigned e = list[t];
-        const long long j = i0 + (e & 0xFFFFu);
-        int c[3];
-        ls_cell(g, j, c);
-        const double r = reinit_r<NDIM>(g, ps, __ldg(p0 + j), thr, c, j, e >> 16);
-        if (mode < 0) out[j] = r;
-        else if (mode == 0) out[j] = ps[j] + dtau * r;
-        else out[j] = 0.5 * pn[j] + 0.5 * (ps[j] + dtau * r);
+    if constexpr (GATHER) {
+        ls_gather(full, threadIdx.x | (need << 16), list, &count);
+        __syncthreads();
+        for (int t = threadIdx.x; t < count; t += kLsThreads) {
+            const unsigned e = list[t];
+            const long long j = i0 + (e & 0xFFFFu);
+            int c[3];
+            ls_cell(g, j, c);
+            put(j, reinit_r<NDIM>(g, ReinitCells<NDIM>(g, ps, c, j), __ldg(p0 + j), thr, e >> 16));
+        }
     }
 }
 
@@ -1289,8 +1316,9 @@ void advect_launch(const LsGrid &g, const double *ps, const double *pn, const do
 void reinit_launch(const LsGrid &g, const double *ps, const double *pn, const double *p0, double thr, double dtau,
                    int mode, double *out, cudaStream_t s) {
     const float lo = std::nextafterf((float)thr, -1.f);  // not above thr
-    if (g.ndim == 3) k_ls_reinit<3><<<ls_blocks(g), kLsThreads, 0, s>>>(g, ps, pn, p0, thr, lo, dtau, mode, out);
-    else k_ls_reinit<2><<<ls_blocks(g), kLsThreads, 0, s>>>(g, ps, pn, p0, thr, lo, dtau, mode, out);
+    auto run = [&](auto kernel) { kernel<<<ls_blocks(g), kLsThreads, 0, s>>>(g, ps, pn, p0, thr, lo, dtau, mode, out); };
+    if (g.ncell > kReinitGather) run(g.ndim == 3 ? k_ls_reinit<3, true> : k_ls_reinit<2, true>);
+    else run(g.ndim == 3 ? k_ls_reinit<3, false> : k_ls_reinit<2, false>);
 }
 
 jxf_status ls_launched() {

@@ -183,3 +183,9 @@ def test_empty_blocks_beside_a_nan(ndim, n, bad):
     jxf.jxf_ls_interface(grid, *W, gamma, pinf, al, dg, nr, want[:ndim], want[ndim])
     jxf.jxf_ls_extend(grid, d, al, dg, nr, want, ndim + 1, 2, 20, z(ndim + 1))
     _same_with_nans(got, want)
+
+
+@pytest.mark.parametrize("amp", [0.0, 0.05, 0.6])
+def test_reinit_screen_is_exact_where_cells_are_gathered(amp):
+    """The same above one block per SM, in the kernel that gathers."""
+    test_reinit_screen_is_exact(3, [37, 35, 33], [(P, P), (Z, S), (S, S)], amp, 1.0 / 64)
