@@ -124,7 +124,10 @@ typedef struct {
  * replaces the CFL step; t_end > 0 clips the last step to end there.
  * eps_rho, eps_rhoc2, eps_alpha <= 0 select the paper's tolerances for the
  * precision (1e-12, 1e-10, 1e-12 in FP64; 1e-10, 1e-8, 1e-10 in FP32);
- * weno_eps <= 0 selects 1e-6.  thinc: THINC reconstruction of the volume
+ * weno_eps <= 0 selects 1e-6.  In FP64 with WENO5, grids above a size (more
+ * faces along an axis than 19456 in 2-D, 38912 / 97280 in single-phase /
+ * five-equation 3-D) evaluate part of a resolved face in pairs of floats: equally
+ * accurate, but rounded otherwise than on smaller grids.  thinc: THINC reconstruction of the volume
  * fraction in interface cells (five-equation model only, §3.2 step 4): a
  * tanh profile fitted to the cell average with steepness |n_d| + 0.01 along
  * axis d (n the normal from the smoothed volume fraction of §3.7), partial

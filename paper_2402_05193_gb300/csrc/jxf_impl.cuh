@@ -157,7 +157,7 @@ struct Dev {
     int teno;    // 1: TENO6-A instead of WENO5
     int viscous, limiter;
     int line_group;  // 1-D grids: lanes per face (see k_line_update)
-    int split;   // double WENO5: resolved faces take the split correction (see kSplitFaces)
+    int split;   // double WENO5: resolved faces take the split correction (see split_faces)
     int visc_half;  // viscous stencils: points per side (1, 2, 3 for order 2, 4, 6)
     int thinc;   // THINC volume-fraction reconstruction (five-equation model)
     double eps_rho, eps_rhoc2, eps_alpha, weno_eps;
@@ -913,13 +913,15 @@ __device__ __forceinline__ void recon_face(const T (&x)[6], T eps4, T &vl, T &vr
 // middle candidate's share of the jump cancels).  The choice is made per face
 // from its own stencil, so it does not depend on how faces are grouped into
 // warps.
-// Small grids (Dev::split = 0: no axis with more faces than one warp for each
-// of the 4 x 152 FP64 pipes, and all 1-D ones) keep the double formula for
-// every face: they are bound by the latency of one warp, and a warp with
-// faces of both kinds pays for both.  us per step, all double | by face: 128^2
-// shock-bubble 231 | 257, 24^3 waves 244 | 320, 200-cell tube 70 | 73.  With the
-// second warp per pipe the double formula takes twice as long: 160^2 bubble
-// 405 | 298, 160^2 waves 254 | 85, 40^3 815 | 295.
+// Small grids (Dev::split = 0; split_faces) and all 1-D ones keep the double
+// formula for every face: up to one warp for each of the 4 x 152 FP64 pipes they are
+// bound by the latency of one warp, and a warp with faces of both kinds pays for
+// both, in 3-D (a third of the warps across x) up to larger sizes.  us per step, all
+// double | by face: 2-D 128^2 shear 191 | 162, shock-bubble 277 | 316; 140^2 (more
+// than a warp per pipe) 294 | 165 and 448 | 323.  3-D single phase, 30^3 waves 471 |
+// 485, vortex 535 | 545; 32^3 472 | 484, 537 | 489; 36^3 (2.5 warps per pipe) 678 | 473,
+// 778 | 701.  3-D five-equation shock-bubble 32^3 702 | 887, 40^3 1330 | 1410, 48^3 (6
+// warps) 1958 | 1917, 64^3 4463 | 3650.  200-cell tube 70 | 73.
 // FP64 instructions of a 3-D viscous face: 620 -> 130; 128^3 Taylor-Green
 // step 24.8 -> 7.6 ms.  Three blocks of 128 an SM (168 registers) let the integer and
 // FP32 work of one warp run beside the FP64 work of the others: 8.75 ms
@@ -1049,7 +1051,13 @@ __device__ __forceinline__ float high_float(unsigned a) {
     return a < 0x38100000u ? 0.f : __uint_as_float(((a << 3) ^ 0x40000000u) & 0x7FFFFFFFu);
 }
 
+// Faces of the axis with most of them from which the choice is made face by
+// face: more than one warp per FP64 pipe, in 3-D two (single phase) or five.  The
+// level-set sweeps, whose warps are sorted by kind, split from one.
 constexpr long long kSplitFaces = 4 * kSMs * 32 + 1;
+constexpr long long split_faces(int model, int ndim) {
+    return ndim < 3 ? kSplitFaces : (model == JXF_DIM ? 5 : 2) * (kSplitFaces - 1) + 1;
+}
 constexpr float kSplitD = 1.f / 16.f;   // bound of |D| over the variable's scale
 constexpr float kSplitT = 1.f / 128.f;  // bound of |T|
 constexpr float kSplitOwn = 1.f / 16.f;  // bound of a transverse velocity's |T| over its largest value

@@ -1574,6 +1574,7 @@ jxf_status jxf_ls_cut_rhs(const jxf_grid *grid, const jxf_eos *eos, const jxf_sc
         return JXF_ERR_UNSUPPORTED;
     jxf::Dev P;
     jxf::fill_dev(grid, eos, scheme, ncell, P);
+    P.split = jxf::split_allowed(grid, P.weno_eps, jxf::kSplitFaces);  // sorted faces: from one warp per pipe
     P.W = const_cast<double *>(W);
     cudaStream_t s = (cudaStream_t)stream;
     const int nv = g.ndim + 2;

@@ -62,6 +62,20 @@ inline jxf_status validate_setup(const jxf_grid *grid, const jxf_eos *eos, const
     return JXF_OK;
 }
 
+// Whether double WENO5 faces choose the split correction: by the whole grid,
+// also for a block of it (the blocks' faces are evaluated as the grid's).  The
+// indicators, at least 4 weno_eps, have to be floats with room for a low part:
+// products of them 2^-48 below still normal numbers.
+inline int split_allowed(const jxf_grid *grid, double weno_eps, long long from) {
+    if (grid->ndim < 2 || !(weno_eps >= 1e-22 && weno_eps <= 1e18)) return 0;
+    for (int d = 0; d < grid->ndim; ++d) {
+        long long nf = 1;
+        for (int e = 0; e < grid->ndim; ++e) nf *= grid->n[e] + (e == d ? 1 : 0);
+        if (nf >= from) return 1;
+    }
+    return 0;
+}
+
 // The grid, material and scheme constants of the kernel parameter block
 // (buffers and scalar slots are left null).
 inline void fill_dev(const jxf_grid *grid, const jxf_eos *eos, const jxf_scheme *scheme,
@@ -130,15 +144,7 @@ inline void fill_dev(const jxf_grid *grid, const jxf_eos *eos, const jxf_scheme 
     P.eps_rhoc2 = scheme->eps_rhoc2 > 0.0 ? scheme->eps_rhoc2 : (f64 ? 1e-10 : 1e-8);
     P.eps_alpha = scheme->eps_alpha > 0.0 ? scheme->eps_alpha : (f64 ? 1e-12 : 1e-10);
     P.weno_eps = scheme->weno_eps > 0.0 ? scheme->weno_eps : 1e-6;
-    // by the whole grid, also for a block of it: the blocks' faces are evaluated
-    // as the grid's.  The indicators, at least 4 weno_eps, have to be floats with
-    // room for a low part: products of them 2^-48 below still normal numbers.
-    const bool eps_fits = P.weno_eps >= 1e-22 && P.weno_eps <= 1e18;
-    for (int d = 0; d < grid->ndim; ++d) {
-        long long nf = 1;
-        for (int e = 0; e < grid->ndim; ++e) nf *= grid->n[e] + (e == d ? 1 : 0);
-        if (grid->ndim > 1 && nf >= kSplitFaces && eps_fits) P.split = 1;
-    }
+    P.split = split_allowed(grid, P.weno_eps, split_faces(eos->model, grid->ndim));
     P.cfl = scheme->cfl;
     P.fixed_dt = scheme->fixed_dt;
     P.t_end = scheme->t_end;

@@ -251,3 +251,19 @@ def test_reverse_sweep_of_uniform_supersonic_flow(weno, recon):
     err = np.abs(got[:, 0] - ref).mean(axis=(1, 2)) / np.abs(ref).mean(axis=(1, 2))
     print(weno, recon, err)
     assert err.max() < 1e-15
+
+
+@pytest.mark.parametrize("recon,weno", [("char", "js"), ("comp", "z")])
+@pytest.mark.parametrize("model,n", [("spm", (138, 139)), ("spm", (139, 140)), ("spm", (33, 34, 33)), ("spm", (36, 34, 32)),
+                                     ("dim", (138, 139)), ("dim", (139, 140)), ("dim", (46, 45, 45)), ("dim", (47, 46, 45))])
+def test_sizes_beside_the_rule(model, n, recon, weno):
+    """Grids below and above the sizes from which faces choose for themselves."""
+    kw = dict(gamma=(1.4, 1.66), rho=(1.2, 0.17), p0=1e5, u0=30.0, limiter=True) if model == "dim" else {}
+    _check(dict(wl.smooth_random(len(n), list(n), model, seed=6, recon=recon, amp=0.02, **kw), weno=weno))
+
+
+@pytest.mark.parametrize("recon,weno", [("char", "js"), ("comp", "z")])
+def test_reverse_sweep_3d_above_the_rule(recon, weno):
+    """As test_reverse_sweep_against_the_oracle_tangent, on a 3-D grid whose
+    faces choose for themselves."""
+    test_reverse_sweep_against_the_oracle_tangent(3, [36, 34, 32], "periodic", 0.02, recon, weno)
