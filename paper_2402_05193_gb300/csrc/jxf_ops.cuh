@@ -43,8 +43,12 @@ inline unsigned grid_for(long long n, int threads) {
 // 33 | 29, 512^2 105 | 79 | 74 | 70 | 78, 1024^2 199 | 178 | 183 | 196 | 231, 32^3
 // viscous 152 | 109 | 90 | 82 | 80, 64^3 183 | 148 | 142 | 140 | 150, 96^3 363 |
 // 333 | 339 | 347 | 383 (chosen: 1, 2, 8, 1, 2, 8).
+// JXF_FUSED_RUN: a fixed run instead, at build time (tuning sweeps).
 constexpr int kFusedRunMax = 16, kFusedBlocks = 5 * kSMs;
 inline int fused_run(const Dev &P, int ndim) {
+#ifdef JXF_FUSED_RUN
+    return JXF_FUSED_RUN;
+#endif
     const long long plane = (long long)P.n[0] * (ndim == 3 ? P.n[1] : 1), n = P.n[ndim - 1];
     int run = kFusedRunMax;
     while (run > 1 && (long long)grid_for(plane, kFluxThreads) * ((n + run - 1) / run) < kFusedBlocks) run /= 2;
