@@ -781,7 +781,6 @@ __device__ __forceinline__ void gather_axis(const Dev &P, const int (&c)[3], T *
     const T *Sbar = static_cast<const T *>(P.Sbar) + sbar_offset(P, NDIM, d, NV);
     // slots hold the adjoint of the mapped cell (mirror flips already applied)
     auto take = [&](int f, int j) {
-#pragma unroll
         const int g = chk_face(P, (long long)f0 + (long long)f * fs, (long long)nface);
 #pragma unroll
         for (int v = 0; v < NV; ++v) acc[v] += Sbar[((size_t)j * NV + v) * nface + (size_t)g];

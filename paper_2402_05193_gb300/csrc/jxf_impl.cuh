@@ -15,7 +15,7 @@
 //               conservation sums and admissibility, reduced per block.
 //   k_aux       one thread per cell: cell-centred velocity gradient of the
 //               new state (viscous) or the THINC interface normal.
-//   k_finalize  one warp: deterministic reduction of the block partials
+//   k_finalize  four warps: deterministic reduction of the block partials
 //               (first folded by k_reduce_partials on large grids), time
 //               advance, next dt (CFL, viscous bound, t_end clip), status
 //               word.
@@ -1700,9 +1700,6 @@ __device__ __forceinline__ void reconstruct_w(const Dev &P, const T (&S)[6][MAXV
     }
 }
 
-// RSV: the kernel variant's scheme family -- 0: WENO5 (Jiang-Shu or Z
-// weights, chosen per face from P.weno_z), 2: TENO6-A (its own kernels, so
-// that its registers do not weigh on the WENO5 sweeps).
 // reconstruct_w() of a double WENO5 face by a group of G neighbouring lanes
 // that hold the same stencil: lane k of the group does the weights of variable
 // k, then all share the values (the same operations, so the same bits).  Where
@@ -1765,6 +1762,9 @@ __device__ __forceinline__ void reconstruct_lanes(const Dev &P, const double (&S
     }
 }
 
+// RSV: the kernel variant's scheme family -- 0: WENO5 (Jiang-Shu or Z
+// weights, chosen per face from P.weno_z), 2: TENO6-A (its own kernels, so
+// that its registers do not weigh on the WENO5 sweeps).
 // HOW a double face is reconstructed: all in double, with the split
 // correction (the caller knows it is resolved), or TRY: TENO6-A with the
 // selection made in float if that is certain, WENO5 split if resolved.
@@ -1895,8 +1895,9 @@ __device__ __forceinline__ void hllc(const Dev &P, const T *WL, const T *WR, T *
 //   phi = (s_K - u)/(s_K - s*) - 1 = a/(s_K - s*),
 //   U* - U = phi rho_k, phi rho w, rho (phi s* + a),
 //            phi E + a ((1 + phi) rho s* + p/(s_K - s*)), phi a1,
-// so 2^-45 of it is far below the rounding of the flux.  About 40 double
-// operations in 3-D instead of 100.  Returns false at s* = 0 (both branches
+// so 2^-46 of a jump of c/128 in the normal velocity (and as much in the
+// pressure) is 2^-53 c, what the rounding of the pressure moves the fluxes by
+// anyway.  About 40 double operations in 3-D instead of 100.  Returns false at s* = 0 (both branches
 // then enter).
 __device__ __forceinline__ f2 rsq2(f2 a) { return mk2(rsq(a.v.x), rsq(a.v.y)); }
 __device__ __forceinline__ d2 drsqrt(d2 x) {  // one correction y (1 - x y^2)/2 of the float estimate
@@ -2401,15 +2402,7 @@ __global__ void __launch_bounds__(kCellThreads, kAuxCells == 4 ? 4 : 6) k_aux_ve
     else grad_vec<NDIM, 2, kAuxCells>(P, (int)q);
 }
 
-// F^d on face i+1/2 of axis d (§2.1): tau_dk and the heat flux from the
-// central stencils of order 2H above -- normal derivative and face value on
-// the normal cells i+1-H..i+H, tangential derivative: the cell-centred
-// derivative (k_aux) of those cells interpolated to the face.  Only du_d/dx_e
-// and du_e/dx_e are needed along a tangential axis e.  S[0..5] are the face's
-// stencil primitives (cells i-2..i+3, boundary-mapped along d, the mirrored
-// normal velocity already flipped); src gives the temperature and the
-// cell-centred derivatives of those cells.
-// The same in double, where every operation counts: normal derivatives and
+// viscous_flux() below in double, where every operation counts: normal derivatives and
 // face velocities from the differences D_k the reconstruction forms anyway,
 //   normal derivative: D2 | 26 D2 - (D1 + D3) |
 //       2134 D2 - 116 (D1 + D3) + 9 (D0 + D4)
@@ -2480,6 +2473,14 @@ __device__ __forceinline__ void viscous_flux_double(const Dev &P, const Src &src
     Fd[1 + NDIM] = fma(C.lam_dn[d], dn[NDIM], work);  // - q_d = + lambda dT/dx_d
 }
 
+// F^d on face i+1/2 of axis d (§2.1): tau_dk and the heat flux from the
+// central stencils of order 2H above -- normal derivative and face value on
+// the normal cells i+1-H..i+H, tangential derivative: the cell-centred
+// derivative (k_aux) of those cells interpolated to the face.  Only du_d/dx_e
+// and du_e/dx_e are needed along a tangential axis e.  S[0..5] are the face's
+// stencil primitives (cells i-2..i+3, boundary-mapped along d, the mirrored
+// normal velocity already flipped); src gives the temperature and the
+// cell-centred derivatives of those cells.
 template <typename T, int NDIM, int d, int H, typename Src>
 __device__ __forceinline__ void viscous_flux(const Dev &P, const Src &src, const T (&S)[6][MAXV], T *Fd) {
     const Cst<T> &C = cst<T>(P);
@@ -2750,7 +2751,7 @@ __device__ __forceinline__ bool flux_one(const Dev &P, double dt, long long g, c
 // with all candidates kept) and the rest; a warp with both runs both codes, one
 // after the other.  TENO6-A, whose long evaluation takes ten times the short
 // one, runs the short one and gathers the block's faces it was not enough for
-// (67x58x45 between walls 1.05 -> 0.89 ms).  SORT (the level-set model, most of
+// (67x58x45 between walls 1.05 -> 0.86 ms).  SORT (the level-set model, most of
 // whose faces are dry and whose interface is lined with unresolved ones): the
 // block sorts its faces beforehand, by integer and float work on the high
 // words, into two lists whose warps are each of one kind, the long ones
@@ -2842,7 +2843,6 @@ __global__ void __launch_bounds__(kFluxThreads, SweepMinBlocks<T, RSV>::value) k
     flux_block<T, MODEL, NDIM, d, VH, RSV, false>(P, dt, base, n, m, true, AllFaces{}, FaceArrays<T, MODEL, NDIM, d>{P, nface});
 }
 
-// -------------------------------------------------- block reductions -----
 // ---------------------------------------------------- shared-memory tiles --
 // The float sweeps across y (and z outside the fused stage) stage the cells
 // of a tile, with three halo cells on each side along the sweep axis, in
