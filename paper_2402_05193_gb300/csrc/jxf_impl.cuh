@@ -1110,6 +1110,21 @@ __device__ __forceinline__ bool split_own(float tm, float big, float c) {
     return tm <= fmaxf(kSplitOwn * big, 5.7e-14f * c);
 }
 
+// Sound speed, density and rho c^2 of a state in float.
+template <int MODEL, int NDIM>
+__device__ __forceinline__ float split_scales(const Cst<float> &C, const float (&w)[Vars<MODEL, NDIM>::NV], float &rho,
+                                              float &rc2) {
+    using V = Vars<MODEL, NDIM>;
+    rho = w[0];
+    if (V::NP == 2) rho += w[V::NP - 1];
+    if (MODEL == JXF_SPM) rc2 = C.gamma0 * (w[V::IE] + C.pinf0);
+    else {
+        const float a1 = w[V::IA >= 0 ? V::IA : 0];
+        rc2 = w[V::IE] + (w[V::IE] + (C.B2h + a1 * C.dBh)) * rcp(C.A2h + a1 * C.dAh);
+    }
+    return rc2 * rsq(rho * rc2);
+}
+
 // Whether a face along axis d takes the split correction: largest |D| and |T|
 // of each variable (dm, tm), the state w2 of cell 2, the largest |x| of each
 // variable (big) and the stencil's largest high word `top` against the bounds;
@@ -1123,14 +1138,8 @@ __device__ __forceinline__ bool split_bounds(const Dev &P, const float (&dm)[Var
     constexpr int NV = V::NV, NP = V::NP, IE = V::IE;
     const Cst<float> &C = P.k32;
     const bool chr = P.recon != JXF_WENO5JS_COMP;
-    float rho = w2[0], rc2;
-    if (NP == 2) rho += w2[NP - 1];
-    if (MODEL == JXF_SPM) rc2 = C.gamma0 * (w2[IE] + C.pinf0);
-    else {
-        const float a1 = w2[V::IA >= 0 ? V::IA : 0];
-        rc2 = w2[IE] + (w2[IE] + (C.B2h + a1 * C.dBh)) * rcp(C.A2h + a1 * C.dAh);
-    }
-    const float c = rc2 * rsq(rho * rc2);
+    float rho, rc2;
+    const float c = split_scales<MODEL, NDIM>(C, w2, rho, rc2);
     bool ok = top < 0x47600000u && rho > 1.5e-5f && rho < 1e10f && rc2 > 1.5e-5f && rc2 < 1e18f && c > 1.5e-5f;
     // 40 max|D|^2 bounds the largest Q; the smallest is at least eps4
     const float qlim = 7e12f * C.weno_eps4;
@@ -1212,6 +1221,8 @@ __device__ __forceinline__ bool reconstruct_split(const Dev &P, const double (&S
 #pragma unroll
     for (int v = 0; v < NV; ++v)
         if (v < NP || v == IE || v == V::IA) split_double(S[2][v], wh[v], wl[v]);
+    float rho, rc2;
+    const float cs = split_scales<MODEL, NDIM>(C, wh, rho, rc2);
     auto largest = [&](int v) {  // largest high word of |x|
         unsigned a = 0;
 #pragma unroll
@@ -1241,7 +1252,7 @@ __device__ __forceinline__ bool reconstruct_split(const Dev &P, const double (&S
                 if (split_across<MODEL, NDIM, d>(v)) {
                     float dm, tm;
                     split_sizes(Dh[0][v], Dh[1][v], Dh[2][v], Dh[3][v], Dh[4][v], dm, tm);
-                    if (!split_own(tm, high_float(largest(v)), 0.f)) {
+                    if (!split_own(tm, high_float(largest(v)), cs)) {
                         weno5_pair_call(z, P.k64.weno_eps4, S[0][v], S[1][v], S[2][v], S[3][v], S[4][v], S[5][v], WL[v], WR[v]);
                         return;
                     }
