@@ -897,11 +897,12 @@ __device__ __forceinline__ void recon_face(const T (&x)[6], T eps4, T &vl, T &vr
 // 2^-4 and |T_k| <= 2^-7 of the variable's scale -- this
 // correction is carried in pairs of floats (an unevaluated sum hi + lo; its
 // error against exact arithmetic is 2^-50 of max |D| in the mean).  The scale is
-// the value itself for densities, partial densities and volume fraction and
-// rho c^2 for the pressure; there the sum with D1 + 2 D2 is in pairs as well (at
-// most 3/16 of the scale).  Velocities cross zero in smooth flow: D up to c/16, T
-// up to c/128, D1 + 2 D2 in double.  The normal one meets the pressure's own
-// rounding, 2^-53 c, in every flux; a transverse one meets nothing but itself,
+// the value itself for densities, partial densities and volume fraction; there
+// the sum with D1 + 2 D2 is in pairs as well (at most 3/16 of the value).
+// Velocities cross zero in smooth flow and a stiffened gas's pressure is small
+// against rho c^2: they are held against c and rho c^2, and D1 + 2 D2 is double.
+// The normal velocity and the pressure meet the pressure's own rounding, 2^-53 c,
+// in every flux; a transverse velocity meets nothing but itself,
 // so its T is also held against its own largest value (kSplitOwn).  Where that
 // fails the face (five-equation model: that velocity) is all double.  The
 // differences and the sum with the cell value, one rounding, are double.
@@ -922,8 +923,8 @@ __device__ __forceinline__ void recon_face(const T (&x)[6], T eps4, T &vl, T &vr
 // 485, vortex 535 | 545; 32^3 472 | 484, 537 | 489; 36^3 (2.5 warps per pipe) 678 | 473,
 // 778 | 701.  3-D five-equation shock-bubble 32^3 702 | 887, 40^3 1330 | 1410, 48^3 (6
 // warps) 1958 | 1917, 64^3 4463 | 3650.  200-cell tube 70 | 73.
-// FP64 instructions of a 3-D viscous face: 620 -> 130; 128^3 Taylor-Green
-// step 24.8 -> 7.6 ms.  Three blocks of 128 an SM (168 registers) let the integer and
+// FP64 instructions of a 3-D viscous face: 620 -> 133; 128^3 Taylor-Green
+// step 24.8 -> 7.8 ms.  Three blocks of 128 an SM (168 registers) let the integer and
 // FP32 work of one warp run beside the FP64 work of the others: 8.75 ms
 // against 9.18 with two and 9.09 with four.
 //
@@ -1247,7 +1248,7 @@ __device__ __forceinline__ bool reconstruct_split(const Dev &P, const double (&S
     };
     auto swp = [](d2 a) { return d2{swap2(a.h), swap2(a.l)}; };
     auto put = [&](int v, d2 o) {
-        if (v >= NP && v < NP + NDIM) {  // velocities cross 0, where D1 + 2 D2 is as large as they are: in double
+        if ((v >= NP && v < NP + NDIM) || v == IE) {  // held against c, rho c^2: D1 + 2 D2 may be as large as they are
             if constexpr (MODEL == JXF_DIM) {
                 if (split_across<MODEL, NDIM, d>(v)) {
                     float dm, tm;
@@ -1264,8 +1265,8 @@ __device__ __forceinline__ bool reconstruct_split(const Dev &P, const double (&S
             WR[v] = fma(-1.0 / 6.0, r - (widen(o.h.v.y) + widen(o.l.v.y)), S[3][v]);
             return;
         }
-        // D1 + 2 D2 less the correction is at most 3/16 of the cell value (of
-        // rho c^2 for the pressure): kept in pairs until the sum with it
+        // D1 + 2 D2 less the correction is at most 3/16 of the cell value: kept in
+        // pairs until the sum with it
         const d2 D2 = pair(2, v);
         const d2 e = renorm(dsub(dadd(pair(1, v), dscale(D2, bc2(2.f))), o));
         WL[v] = fma(1.0 / 6.0, widen(e.h.v.x) + widen(e.l.v.x), S[2][v]);
